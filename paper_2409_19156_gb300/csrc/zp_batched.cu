@@ -32,6 +32,7 @@
 #include "zp_api_common.h"
 #include "zp_fused.h"
 #include "zp_series_internal.h"
+#include "zp_tri_host.h"
 
 namespace zp {
 namespace {
@@ -426,6 +427,14 @@ struct zp_batch {
   zp::FusedItem* d_fitems = nullptr;
   int32_t* d_fchunk = nullptr;
   int64_t n_fitems = 0, n_fchunks = 0;
+  // The triangle form of the same launches, when every instance's plan has that layout: descriptors
+  // of the values, then of the gradients, sharing items, digits and scales.
+  bool tri_ok = false;
+  void* tri_block = nullptr;
+  zp::TriInst* d_tinst = nullptr;
+  int32_t* d_tchunk = nullptr;
+  int64_t n_tchunks = 0;
+  int tri_n_max = 0;
   int fused_ndig = zp::kFusedDigits;  // digits per value of the fused launches (the longest instance's)
 };
 
@@ -619,7 +628,75 @@ zp_status build_fused(zp_batch* b) {
   return ZP_OK;
 }
 
+// Descriptors and buffers of the triangle form (see zp_batch::tri_ok).  Without the memory for
+// them the batch keeps the column form.
+zp_status build_tri(zp_batch* b) {
+  if (!b->fused_ok) return ZP_OK;
+  const int64_t n = (int64_t)b->inst.size();
+  bool grads = false;
+  for (int64_t i = 0; i < n; ++i) {
+    if (b->inst[i].n_modes == 0) continue;
+    const zp_plan* p = b->plans[b->inst_plan[i]].get();
+    if (!p->tri) return ZP_OK;
+    b->tri_n_max = std::max(b->tri_n_max, p->n_max);
+    grads |= b->inst[i].grad_r || b->inst[i].grad_theta;
+  }
+  std::vector<TriInst> ti(2 * n);
+  std::vector<int32_t> chunk_inst;
+  for (int64_t i = 0; i < n; ++i) {
+    const zp_instance& in = b->inst[i];
+    if (in.n_modes == 0) continue;
+    TriInst& d = ti[i];
+    d = tri_inst(b->plans[b->inst_plan[i]].get(), in.r, in.theta, in.n_points, in.coeffs, b->n_sets);
+    d.kc_base = (int64_t)chunk_inst.size();
+    d.out = (double*)in.out;
+    chunk_inst.insert(chunk_inst.end(), d.KC, (int32_t)i);
+  }
+  const int64_t chunks = (int64_t)chunk_inst.size();
+  if (chunks == 0) return ZP_OK;
+  const size_t inst_b = align256(2 * n * sizeof(TriInst)), chunk_b = align256(chunks * sizeof(int32_t));
+  const size_t cexp_b = align256(2 * n * kFusedMaxSets * sizeof(int));
+  const size_t dig_b = tri_digit_bytes(chunks, grads), cpos_b = grads ? tri_cpos_bytes(chunks) : 0;
+  if (cudaMalloc(&b->tri_block, inst_b + chunk_b + cexp_b + dig_b + cpos_b) != cudaSuccess) {
+    cudaGetLastError();
+    b->tri_block = nullptr;
+    return ZP_OK;
+  }
+  char* base = (char*)b->tri_block;
+  const int groups = grads ? 2 : 1;
+  for (int64_t i = 0; i < n; ++i) {
+    const zp_instance& in = b->inst[i];
+    TriInst& d = ti[i];
+    if (in.n_modes == 0) continue;
+    d.cexp = (int*)(base + inst_b + chunk_b) + 2 * i * kFusedMaxSets;
+    d.bdig = (uint8_t*)(base + inst_b + chunk_b + cexp_b) + (size_t)d.kc_base * kTriGroupBytes;
+    TriInst& g = ti[n + i];
+    g = d;
+    g.bdig = (uint8_t*)(base + inst_b + chunk_b + cexp_b) + (size_t)d.kc_base * kTriGroupBytes * groups;
+    g.cpos = grads ? (double*)(base + inst_b + chunk_b + cexp_b + dig_b) + 2 * d.kc_base * kTriChunk * kFusedMaxSets : nullptr;
+    g.out = nullptr;
+    g.gdot = in.grad_out;
+    g.grad_r = in.grad_r;
+    g.grad_theta = in.grad_theta;
+  }
+  b->d_tinst = (TriInst*)base;
+  b->d_tchunk = (int32_t*)(base + inst_b);
+  b->n_tchunks = chunks;
+  cudaError_t e = cudaMemcpy(b->d_tinst, ti.data(), 2 * n * sizeof(TriInst), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_tchunk, chunk_inst.data(), chunks * sizeof(int32_t), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return cuda_error(e, "copy of triangle batch descriptors");
+  b->tri_ok = true;
+  return ZP_OK;
+}
+
 zp_status batch_forward(zp_batch* b, zp_precision prec, cudaStream_t st) {
+  if (prec == ZP_PREC_FP64_EMULATED && b->tri_ok) {
+    TriArgs a;
+    a.insts = b->d_tinst;
+    a.items = b->d_fitems;
+    a.n_items = b->n_fitems;
+    return tri_launch(a, b->tri_n_max, b->d_tchunk, b->n_tchunks, false, st);
+  }
   if (prec == ZP_PREC_FP64_EMULATED) {
     if (!b->fused_ok)
       return set_error(ZP_ERR_UNSUPPORTED, "the emulated float64 batched forward takes at most 16 sets and 5041 "
@@ -702,7 +779,7 @@ zp_status zp_batch_create(const zp_instance* instances, int64_t n_instances, int
   for (auto& p : b->plans) {
     size_t o6[kPlanSections];
     plan_off.push_back(off);
-    off += align256(plan_device_layout(p.get(), o6));
+    off += align256(plan_device_layout(p.get(), o6)) + plan_tri_bytes(p.get());
   }
   const size_t desc_off = off;
   off += align256(std::max<int64_t>(n_instances, 1) * sizeof(InstanceDesc));
@@ -729,7 +806,10 @@ zp_status zp_batch_create(const zp_instance* instances, int64_t n_instances, int
   if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(batch)");
   char* base = (char*)b->dev_block;
   for (size_t k = 0; k < b->plans.size(); ++k) {
-    zp_status st = plan_upload(b->plans[k].get(), base + plan_off[k], nullptr, false);
+    size_t o6[kPlanSections];
+    zp_plan* p = b->plans[k].get();
+    zp_status st = plan_upload(p, base + plan_off[k], nullptr, false);
+    if (st == ZP_OK) st = plan_tri_upload(p, base + plan_off[k] + align256(plan_device_layout(p, o6)));
     if (st != ZP_OK) {
       cudaFree(b->dev_block);
       return st;
@@ -789,9 +869,11 @@ zp_status zp_batch_create(const zp_instance* instances, int64_t n_instances, int
   zp_status st = build_point_items(b.get(), nullptr);
   if (st == ZP_OK) st = set_column_attributes(b.get());
   if (st == ZP_OK) st = build_fused(b.get());
+  if (st == ZP_OK) st = build_tri(b.get());
   if (st != ZP_OK) {
     cudaFree(b->dev_block);
     if (b->fused_block) cudaFree(b->fused_block);
+    if (b->tri_block) cudaFree(b->tri_block);
     return st;
   }
   *out = b.release();
@@ -807,6 +889,7 @@ zp_status zp_batch_destroy(zp_batch* b) {
   cudaDeviceSynchronize();
   if (b->dev_block) cudaFree(b->dev_block);
   if (b->fused_block) cudaFree(b->fused_block);
+  if (b->tri_block) cudaFree(b->tri_block);
   cudaSetDevice(cur);
   delete b;
   return ZP_OK;
@@ -879,7 +962,14 @@ static zp_status zp_batch_adjoint_impl(zp_batch* b, zp_precision prec, void* str
     if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
   }
   if (b->n_sets == 0) return ZP_OK;
-  if (need_pt && prec == ZP_PREC_FP64_EMULATED && b->fused_ok) {
+  if (need_pt && prec == ZP_PREC_FP64_EMULATED && b->tri_ok) {
+    // Both point gradients in one pass over the points: the series of dF/dx and dF/dy.
+    TriArgs a;
+    a.insts = b->d_tinst + b->inst.size();
+    a.items = b->d_fitems;
+    a.n_items = b->n_fitems;
+    ZP_TRY(tri_launch(a, b->tri_n_max, b->d_tchunk, b->n_tchunks, true, st));
+  } else if (need_pt && prec == ZP_PREC_FP64_EMULATED && b->fused_ok) {
     // grad_theta[p] = sum_s G[p][s] (dZ/dtheta C)[p][s] and grad_r likewise with dZ/drho: the
     // fused tensor-core kernel for the two derivative series, each row sum formed in its drain
     // and added onto the zeroed gradients.

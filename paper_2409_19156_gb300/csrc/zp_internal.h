@@ -73,6 +73,7 @@ struct DevicePlanTables {
   int32_t* mode_col = nullptr;  // [n_modes]: column index of every mode
   int32_t* mode_N = nullptr;    // [n_modes]: Jacobi degree of every mode
   uint2* split_step = nullptr;  // [table rows]: step descriptors of the split basis
+  int32_t* tri_perm = nullptr;  // [tri_chunks * 16]: mode of every triangle position, -1 for none (plans with tri)
   int4* fused_col = nullptr;    // [columns]: fused contraction layout (see kFusedKind*)
   int32_t* fused_kperm = nullptr;  // [fused_kpad]: slot of every K position, -1 for padding
 };
@@ -95,6 +96,8 @@ struct zp_plan {
   int32_t fused_ncols[zp::kFusedStreams] = {};  // columns per stream
   int32_t fused_units = 0;  // global 8-value units G of the layout (whole 4-unit stages); stream s owns (G - s + S - 1) / S
   int32_t fused_ep = 1;              // row scale exponent of the fused kernel on the unit disc
+  bool tri = false;                  // the mode list suits the triangle layout (zp_tri.h)
+  std::vector<int32_t> tri_perm;     // its positions' modes (empty without it)
   zp::DevicePlanTables dev;
   size_t device_bytes = 0;
   void* dev_block = nullptr;  // single allocation backing dev.*
@@ -118,6 +121,10 @@ size_t plan_device_layout(const zp_plan* p, size_t offsets[kPlanSections]);
 // Points p->dev at `base` (laid out as plan_device_layout) and copies the host tables there,
 // with cudaMemcpyAsync on `stream` when async, else synchronously.
 zp_status plan_upload(zp_plan* p, void* base, cudaStream_t stream, bool async);
+// The triangle layout's table, kept behind that block by plans that own their device memory: its
+// size in bytes (a multiple of 256, 0 without the layout) and its upload (synchronous).
+size_t plan_tri_bytes(const zp_plan* p);
+zp_status plan_tri_upload(zp_plan* p, void* base);
 // Cached plan for a mode list on the current device (created on first use).  The caller
 // keeps *out alive while it uses the plan; the cache may drop its own reference.
 zp_status cached_plan(const int32_t* n, const int32_t* m, int64_t n_modes, std::shared_ptr<const zp_plan>* out);

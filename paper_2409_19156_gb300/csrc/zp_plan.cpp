@@ -19,6 +19,7 @@
 #include <unordered_map>
 
 #include "zp_internal.h"
+#include "zp_tri.h"
 
 namespace zp {
 
@@ -275,6 +276,24 @@ zp_status build_plan_host(const int32_t* n, const int32_t* m, int64_t n_modes, z
   int e = 0;
   while (std::ldexp(1.0, e) <= inv_w * (1.0 + 1e-9)) ++e;
   p->fused_ep = e;
+  // Triangle layout: every (n, |m|) with n <= n_max gets a cos and a sin position, so it suits mode
+  // lists without duplicates that fill enough of their triangle.  A full list has about as many
+  // positions in either layout, and there the triangle form takes 0.60 of the column form's time
+  // (n <= 32, 1e6 points, 16 sets: 2.37 against 3.91 ms), so lists whose triangle has up to half as
+  // many positions again still gain.
+  if (n_modes > 0 && n_max <= kTriMaxN) {
+    const int64_t positions = (int64_t)tri_chunks(n_max) * kTriChunk;
+    if (2 * positions <= 3 * p->fused_kpad) {
+      p->tri_perm.assign((size_t)positions, -1);
+      p->tri = true;
+      for (int64_t j = 0; j < n_modes && p->tri; ++j) {
+        int32_t& at = p->tri_perm[tri_position(n[j], std::abs(m[j]), m[j] < 0 ? 1 : 0, n_max)];
+        p->tri = at < 0;
+        at = (int32_t)j;
+      }
+      if (!p->tri) p->tri_perm.clear();
+    }
+  }
   return ZP_OK;
 }
 
@@ -336,17 +355,27 @@ zp_status plan_upload(zp_plan* p, void* base_ptr, cudaStream_t stream, bool asyn
   return ZP_OK;
 }
 
+size_t plan_tri_bytes(const zp_plan* p) { return align_up(p->tri_perm.size() * sizeof(int32_t), 256); }
+
+zp_status plan_tri_upload(zp_plan* p, void* base) {
+  if (!p->tri) return ZP_OK;
+  p->dev.tri_perm = (int32_t*)base;
+  const cudaError_t e = cudaMemcpy(base, p->tri_perm.data(), p->tri_perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? ZP_OK : cuda_error(e, "copy of plan tables");
+}
+
 zp_status build_plan(const int32_t* n, const int32_t* m, int64_t n_modes, zp_plan** out) {
   if (!out) return set_error(ZP_ERR_INVALID_ARG, "plan output pointer is NULL");
   std::unique_ptr<zp_plan> p(new zp_plan());
   zp_status st = build_plan_host(n, m, n_modes, p.get());
   if (st != ZP_OK) return st;
   size_t off[kPlanSections];
-  const size_t total = plan_device_layout(p.get(), off);
+  const size_t tri_off = plan_device_layout(p.get(), off), total = tri_off + plan_tri_bytes(p.get());
   cudaError_t e = cudaMalloc(&p->dev_block, total);
   if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(plan tables)");
   p->device_bytes = total;
   st = plan_upload(p.get(), p->dev_block, nullptr, false);
+  if (st == ZP_OK) st = plan_tri_upload(p.get(), (char*)p->dev_block + tri_off);
   if (st != ZP_OK) {
     cudaFree(p->dev_block);
     return st;

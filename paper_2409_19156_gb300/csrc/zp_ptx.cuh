@@ -99,6 +99,32 @@ __device__ __forceinline__ bool mbar_wait_sleepy(uint64_t* bar, uint32_t parity,
   }
 }
 
+// mbar_wait whose polls let the hardware suspend the thread for up to about a microsecond each,
+// so that a waiting thread takes no issue slots and still wakes as soon as the phase completes.
+__device__ __forceinline__ bool mbar_wait_suspend(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                  uint64_t limit_ns = kWaitLimitNs) {
+  auto poll = [&]() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(1000u)
+        : "memory");
+    return ok != 0;
+  };
+  if (poll()) return true;
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t i = 0;; ++i) {
+    if (poll()) return true;
+    if ((i & 15u) == 15u) {
+      if (*abort_flag) return false;
+      if (global_timer_ns() - t0 > limit_ns) return false;
+    }
+  }
+}
+
 // Bulk copy global -> shared, completing `bytes` transaction bytes on `bar`.
 __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
   asm volatile(
@@ -166,12 +192,12 @@ __device__ __forceinline__ void tc_fence_after() {
 }
 
 // Shared-memory matrix descriptor: K-major operand in the ROW-byte swizzle layout (rows of ROW
-// bytes, 8-row groups 8 * ROW bytes apart; ROW = 128 or 64), descriptor version 1.  Layout
-// field: 2 = 128-byte swizzle, 4 = 64-byte swizzle.
+// bytes, 8-row groups 8 * ROW bytes apart; ROW = 128, 64 or 32), descriptor version 1.  Layout
+// field: 2 = 128-byte swizzle, 4 = 64-byte swizzle, 6 = 32-byte swizzle.
 template <uint32_t ROW>
 __device__ __forceinline__ uint64_t sw_kmajor_desc(uint32_t saddr) {
-  static_assert(ROW == 128 || ROW == 64, "128- or 64-byte swizzle");
-  constexpr uint64_t layout = ROW == 128 ? 2u : 4u;
+  static_assert(ROW == 128 || ROW == 64 || ROW == 32, "128-, 64- or 32-byte swizzle");
+  constexpr uint64_t layout = ROW == 128 ? 2u : (ROW == 64 ? 4u : 6u);
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)((8u * ROW) >> 4) << 32) |
          ((uint64_t)1 << 46) | (layout << 61);
 }
@@ -179,6 +205,10 @@ __device__ __forceinline__ uint64_t sw_kmajor_desc(uint32_t saddr) {
 // Instruction descriptor for kind::f16 (A, B = bf16; D = f32; both K-major).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+// Instruction descriptor for kind::f16 (A, B = float16; D = f32; both K-major).
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // Instruction descriptor for kind::tf32 (A, B = tf32; D = f32; both K-major).
 __host__ __device__ constexpr uint32_t idesc_tf32_f32(int M, int N) {
@@ -192,6 +222,18 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same with A in tensor memory: row i in lane i, 16-bit elements 2c and 2c + 1 of the K step
+// in column c from a_tmem.
+__device__ __forceinline__ void mma_f16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -282,6 +324,17 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[8]) {
                : "memory");
 }
 
+// 32 lanes x 4 consecutive 32-bit columns at taddr + OFFSET: thread i of the warp writes lane (base
+// lane + i).
+template <int OFFSET>
+__device__ __forceinline__ void tmem_st_32x32b_x4(uint32_t taddr, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0 + %5], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v0), "r"(v1),
+               "r"(v2), "r"(v3), "n"(OFFSET)
+               : "memory");
+}
+// Waits for this thread's tcgen05.st stores.
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // Makes this thread's generic-proxy shared-memory writes visible to the async proxy (the
 // tensor core reading operands through matrix descriptors); issue before the mbarrier arrive
 // that hands the data over.
@@ -291,14 +344,17 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 
 // Physical 16-byte unit of logical unit `unit` in row `row` of a K-major tile in the ROW-byte
 // swizzle layout: 128 bytes XOR the unit index (3 bits) with row % 8; 64 bytes XOR it (2 bits)
-// with (row / 2) % 4 (address bits 6:4 with 9:7, resp. 5:4 with 8:7).
+// with (row / 2) % 4; 32 bytes XOR it (1 bit) with (row / 4) % 2 (address bits 6:4 with 9:7,
+// resp. 5:4 with 8:7, resp. 4 with 7).
 template <uint32_t ROW>
 __host__ __device__ __forceinline__ uint32_t sw_unit(uint32_t row, uint32_t unit) {
-  static_assert(ROW == 128 || ROW == 64, "128- or 64-byte swizzle");
+  static_assert(ROW == 128 || ROW == 64 || ROW == 32, "128-, 64- or 32-byte swizzle");
   if constexpr (ROW == 128) {
     return unit ^ (row & 7u);
-  } else {
+  } else if constexpr (ROW == 64) {
     return unit ^ ((row >> 1) & 3u);
+  } else {
+    return unit ^ ((row >> 2) & 1u);
   }
 }
 // Byte offset of element (row, k) of a K-major tile of 2-byte elements (ROW / 2 per row; the

@@ -21,6 +21,7 @@
 #include "zp_api_common.h"
 #include "zp_fused.h"
 #include "zp_series_internal.h"
+#include "zp_tri_host.h"
 
 namespace zp {
 namespace {
@@ -274,7 +275,10 @@ zp_status series_adjoint_fp64(const zp_plan* plan, const double* r, const double
   // derivative series (no [modes x points] H).
   const bool fused_pt = emulated && !ho.any() && (grad_r || grad_theta) && S <= kFusedMaxSets &&
                         plan->fused_kpad <= kFusedMaxModes;
-  if (fused_pt) ZP_TRY(fused_point_grads(plan, r, theta, P, coeffs, S, G, grad_r, grad_theta, stream));
+  if (fused_pt && plan->tri)
+    ZP_TRY(tri_point_grads(plan, r, theta, P, coeffs, S, G, grad_r, grad_theta, stream));
+  else if (fused_pt)
+    ZP_TRY(fused_point_grads(plan, r, theta, P, coeffs, S, G, grad_r, grad_theta, stream));
   const bool need_h = !fused_pt && (grad_r || grad_theta || ho.any());
   ScratchBuffer z, hbuf;
   CublasLock cl;
@@ -361,6 +365,8 @@ static zp_status zp_series_eval_plan_impl(const zp_plan* plan, const double* r, 
   if (prec == ZP_PREC_FP64) return series_eval_fp64(plan, r, theta, n_points, coeffs, n_sets, (double*)out, st);
   if (prec == ZP_PREC_FP64_EMULATED) {
     // Few sets: the fused kernel (basis generated on chip, no basis or partial sums in HBM).
+    if (n_sets <= kFusedMaxSets && plan->tri)
+      return tri_series_eval(plan, r, theta, n_points, coeffs, n_sets, (double*)out, st);
     if (n_sets <= kFusedMaxSets && plan->fused_kpad <= kFusedMaxModes)
       return fused_series_eval(plan, r, theta, n_points, coeffs, n_sets, (double*)out, st);
     return series_eval_emulated_fp64(plan, r, theta, n_points, coeffs, n_sets, (double*)out, st);

@@ -9,6 +9,7 @@
 
 #include "zp_api_common.h"
 #include "zp_fused.h"
+#include "zp_tri_host.h"
 
 namespace zp {
 
@@ -38,8 +39,9 @@ zp_status entry_finish(const char* name, void* stream, zp_status st) {
       if (e != cudaSuccess) {
         st = cuda_error(e, what.c_str());
       } else {
-        unsigned int a = 0, b = 0;
-        if (split_error_word(&a, false) == ZP_OK && fused_error_word(&b, false) == ZP_OK && (a || b))
+        unsigned int a = 0, b = 0, c = 0;
+        if (split_error_word(&a, false) == ZP_OK && fused_error_word(&b, false) == ZP_OK &&
+            tri_error_word(&c, false) == ZP_OK && (a || b || c))
           st = set_error(ZP_ERR_TIMEOUT, what + ": a bounded device wait gave up");
       }
     } else {
