@@ -654,8 +654,8 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
             l1 = begin ? kTriZero : l1;
             dg = begin ? (bi.A == 0 ? 0ull : kTriZero) : dg;
             const uint64_t u0 = diag ? l0 : s0, u1 = diag ? l1 : s1;
-            const uint64_t e00 = tri_step(tp, u0, l0, dg), e01 = tri_step(tp, u1, e00, u0);
-            const uint64_t e10 = tri_step(tp, e00, l1, l0), e11 = tri_step(tp, e01, e10, e00);
+            const uint64_t e00 = tri_floor(tri_step(tp, u0, l0, dg)), e01 = tri_step(tp, u1, e00, u0);
+            const uint64_t e10 = tri_step(tp, e00, l1, l0), e11 = tri_floor(tri_step(tp, e01, e10, e00));
             r[0] = e10;
             r[TM] = e11;
             f[(size_t)(4 * k) * TM] = e00;

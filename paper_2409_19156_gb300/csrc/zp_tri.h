@@ -27,6 +27,7 @@
 namespace zp {
 
 constexpr int kTriMaxN = 64;      // largest n_max (shared memory for a tile's state and angles)
+constexpr int kTriMaxWalkN = 256; // largest n_max of the float64 walk over the same layout
 constexpr int kTriDigits = 9;     // base-64 digits per value
 constexpr int kTriChunk = 16;     // positions per chunk (one tensor-core K step)
 // Longest run of positions whose diagonal sums stay below 2^24 (exact in float32): digits of at
@@ -137,14 +138,19 @@ __host__ __device__ __forceinline__ uint64_t tri_step(const TriPoint& t, uint64_
   return tri_mul_add(f1 + f2, t.rho, t.bias - f0);
 }
 
+// A biased word kept from wrapping below -1: R_n^0 comes that close near the origin (n = 2 mod 4), and
+// tri_word takes the word as unsigned.  Only m = 0 needs it: elements e00 and e11.
+__host__ __device__ __forceinline__ uint64_t tri_floor(uint64_t f) { return (int64_t)f < 0 ? 0 : f; }
+
 // A signed number of [-1, 1] at scale 2^62 as a high word (31 bits down) and 31 low bits.
 struct TriTrig {
   int32_t hi;
   uint32_t lo;
 };
 __host__ __device__ __forceinline__ TriTrig tri_split(int64_t v) {
-  const int64_t top = (1ll << 62) - 1;
-  v = v > top ? top : v;
+  // Rounding may carry a cosine of +-1 just beyond the range.
+  const int64_t top = (1ll << 62) - 1, bottom = -(1ll << 62);
+  v = v > top ? top : (v < bottom ? bottom : v);
   TriTrig t;
   t.hi = (int32_t)(v >> 31);
   t.lo = (uint32_t)v & 0x7fffffffu;

@@ -29,11 +29,14 @@ def driver(tmp_path_factory):
 
 @pytest.mark.parametrize("n_max", [0, 1, 2, 3, 7, 32, 33, 64])
 def test_walk_against_oracle(driver, n_max):
-    r, th = inputs.uniform_points(8, 40 + n_max)
-    r[:3], th[:4] = [0.0, 1.0, 1e-3], [0.0, np.pi, -1900.0, 1e-12]
+    # Random angles, and those whose multiples meet the axes, where cos and sin reach +-1.
+    r, th = inputs.uniform_points(40, 40 + n_max)
+    r[:3], th[:4], th[4:28] = [0.0, 1.0, 1e-3], [0.0, np.pi, -1900.0, 1e-12], np.arange(24) * (np.pi / 12)
+    # Radii at which R_n^0 rounds to -1, where the biased words end.
+    r[28:40] = [1e-4, 1e-6, 1e-8, 3e-9, 1e-9, 1e-10, 1e-12, 1e-15, 1e-18, 5e-20, 1e-30, 1e-300]
     text = "".join(f"{float(a).hex()} {float(b).hex()}\n" for a, b in zip(r, th))
     out = subprocess.run([driver, str(n_max)], input=text, capture_output=True, text=True, check=True).stdout
-    got = np.array([line.split() for line in out.splitlines()], dtype=np.int64).reshape(8, -1, 3)
+    got = np.array([line.split() for line in out.splitlines()], dtype=np.int64).reshape(40, -1, 3)
     ns, ms = got[0, :, 0], got[0, :, 1]
     want = np.array(obasis.basis_table(ns, ms, r, th, 0)[0][0]).T
     # Half a unit of the last digit, the oracle's own rounding, two units of 2^-61 from each of the
@@ -86,3 +89,33 @@ def test_series_and_gradients_against_the_baseline(n_max, P, S, which):
         bounds.append(1e-13 * (G.abs() * (1.0 + (d.abs() + n2).T @ C.abs())).sum(1))
     for g, w, b in zip(got, want, bounds):
         assert bool(((g - w).abs() <= b).all()), float(((g - w).abs() / b).max())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_max,k,which", [(2, 3, "full"), (9, 0, "full"), (16, 2, "most"), (33, 1, "full"), (100, 3, "radial"),
+                                           (101, 0, "radial")])
+def test_float64_walk_against_oracle(n_max, k, which):
+    """Enough points for whole waves of the triangle form and a rest for the column form; points of
+    both, at the edges of blocks and waves, at the origin, the rim, a small angle and off the disc."""
+    torch = pytest.importorskip("torch")
+    import paper_2409_19156_gb300 as zp
+    from oracle import radial as oradial
+
+    P = 40_001
+    ns, ms = inputs.radial_modes(n_max) if which == "radial" else _lists(n_max, which)
+    r, th = inputs.uniform_points(P, n_max)
+    rows = np.array([0, 1, 31, 32, 19_455, 19_456, 38_911, 38_912, 40_000])
+    r[[0, 1, 32]], th[[31, 32]] = [0.0, 1.0, 1.02], [1e-9, -2500.0]
+    if which != "radial":
+        th[rows] = np.clip(th[rows], -3.0, 3.0)
+    rt, tt = (torch.as_tensor(x, device="cuda") for x in (r, th))
+    tol = 1e-11 * np.maximum(ns, 1).astype(float)[None, :, None] ** (2 * np.arange(k + 1))[:, None, None]
+    if which == "radial":
+        got = zp.radial(ns, ms, rt, k)[:, :, rows].cpu().numpy()
+        want = np.array(oradial.radial_table(ns, ms, r[rows], k))
+    else:
+        got, dt = (x[..., rows].cpu().numpy() for x in zp.basis(ns, ms, rt, tt, k, dtheta=True))
+        want, wt = obasis.basis_table(ns, ms, r[rows], th[rows], k, with_dtheta=True)
+        assert (np.abs(dt - np.array(wt)) <= 1e-11 * np.maximum(ns, 1)[:, None] * 1.02 ** ns[:, None]).all()
+    far = np.where(r[rows] > 1.0, 8.0 ** np.minimum(n_max, 12), 1.0)  # values beyond the rim grow past 1
+    assert (np.abs(got - np.array(want)) <= tol * far).all()

@@ -49,8 +49,8 @@ int main(int, char** argv) {
       uint64_t l0 = kTriZero, l1 = kTriZero, dg = A == 0 ? 0 : kTriZero;
       for (int B = 0; B <= (A < H - A ? A : H - A); ++B, ++i) {
         const uint64_t u0 = B < A ? st[2 * B] : l0, u1 = B < A ? st[2 * B + 1] : l1;
-        const uint64_t e00 = tri_step(tp, u0, l0, dg), e01 = tri_step(tp, u1, e00, u0);
-        const uint64_t e10 = tri_step(tp, e00, l1, l0), e11 = tri_step(tp, e01, e10, e00);
+        const uint64_t e00 = tri_floor(tri_step(tp, u0, l0, dg)), e01 = tri_step(tp, u1, e00, u0);
+        const uint64_t e10 = tri_step(tp, e00, l1, l0), e11 = tri_floor(tri_step(tp, e01, e10, e00));
         st[2 * B] = e10;
         st[2 * B + 1] = e11;
         dg = u1;
