@@ -73,7 +73,7 @@ struct DevicePlanTables {
   int32_t* mode_col = nullptr;  // [n_modes]: column index of every mode
   int32_t* mode_N = nullptr;    // [n_modes]: Jacobi degree of every mode
   uint2* split_step = nullptr;  // [table rows]: step descriptors of the split basis
-  int32_t* tri_perm = nullptr;  // [tri_chunks * 16]: mode of every triangle position, -1 for none (plans with tri)
+  int32_t* tri_perm = nullptr;  // [tri_chunks * 16]: mode of every triangle position, -1 for none; NULL without the layout
   int4* fused_col = nullptr;    // [columns]: fused contraction layout (see kFusedKind*)
   int32_t* fused_kperm = nullptr;  // [fused_kpad]: slot of every K position, -1 for padding
 };
@@ -96,8 +96,8 @@ struct zp_plan {
   int32_t fused_ncols[zp::kFusedStreams] = {};  // columns per stream
   int32_t fused_units = 0;  // global 8-value units G of the layout (whole 4-unit stages); stream s owns (G - s + S - 1) / S
   int32_t fused_ep = 1;              // row scale exponent of the fused kernel on the unit disc
-  bool tri = false;                  // the mode list suits the triangle layout (zp_tri.h)
-  std::vector<int32_t> tri_perm;     // its positions' modes (empty without it)
+  bool tri = false;                  // the fused series takes the triangle layout (zp_tri.h)
+  std::vector<int32_t> tri_perm;     // the layout's positions' modes (empty without it)
   zp::DevicePlanTables dev;
   size_t device_bytes = 0;
   void* dev_block = nullptr;  // single allocation backing dev.*

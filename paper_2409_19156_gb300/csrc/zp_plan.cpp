@@ -276,23 +276,29 @@ zp_status build_plan_host(const int32_t* n, const int32_t* m, int64_t n_modes, z
   int e = 0;
   while (std::ldexp(1.0, e) <= inv_w * (1.0 + 1e-9)) ++e;
   p->fused_ep = e;
-  // Triangle layout: every (n, |m|) with n <= n_max gets a cos and a sin position, so it suits mode
-  // lists without duplicates that fill enough of their triangle.  A full list has about as many
-  // positions in either layout, and there the triangle form takes 0.60 of the column form's time
-  // (n <= 32, 1e6 points, 16 sets: 2.37 against 3.91 ms), so lists whose triangle has up to half as
-  // many positions again still gain.
-  if (n_modes > 0 && n_max <= kTriMaxN) {
+  // Triangle layout: every (n, |m|) with n <= n_max gets a cos and a sin position, for mode lists
+  // without duplicates that fill at least half of the (n, |m|) of their triangle.
+  std::vector<char> pair_seen(n_max <= kTriMaxWalkN ? (size_t)(n_max + 1) * (n_max + 1) : 0, 0);
+  int64_t pairs = 0;
+  for (int64_t j = 0; j < n_modes && !pair_seen.empty(); ++j) {
+    char& seen = pair_seen[(size_t)n[j] * (n_max + 1) + std::abs(m[j])];
+    pairs += seen == 0;
+    seen = 1;
+  }
+  if (n_modes > 0 && 2 * pairs >= (int64_t)(n_max / 2 + 1) * ((n_max + 1) / 2 + 1)) {
     const int64_t positions = (int64_t)tri_chunks(n_max) * kTriChunk;
-    if (2 * positions <= 3 * p->fused_kpad) {
-      p->tri_perm.assign((size_t)positions, -1);
-      p->tri = true;
-      for (int64_t j = 0; j < n_modes && p->tri; ++j) {
-        int32_t& at = p->tri_perm[tri_position(n[j], std::abs(m[j]), m[j] < 0 ? 1 : 0, n_max)];
-        p->tri = at < 0;
-        at = (int32_t)j;
-      }
-      if (!p->tri) p->tri_perm.clear();
+    p->tri_perm.assign((size_t)positions, -1);
+    bool once = true;
+    for (int64_t j = 0; j < n_modes && once; ++j) {
+      int32_t& at = p->tri_perm[tri_position(n[j], std::abs(m[j]), m[j] < 0 ? 1 : 0, n_max)];
+      once = at < 0;
+      at = (int32_t)j;
     }
+    if (!once) p->tri_perm.clear();
+    // The fused series also wants enough of the positions taken.  A full list has about as many in
+    // either layout, and there the triangle form takes 0.60 of the column form's time (n <= 32, 1e6
+    // points, 16 sets: 2.37 against 3.91 ms), so up to half as many positions again still gain.
+    p->tri = once && n_max <= kTriMaxN && 2 * positions <= 3 * p->fused_kpad;
   }
   return ZP_OK;
 }
@@ -332,33 +338,35 @@ zp_status plan_upload(zp_plan* p, void* base_ptr, cudaStream_t stream, bool asyn
   p->dev.fused_col = (int4*)(base + off[7]);
   p->dev.fused_kperm = (int32_t*)(base + off[8]);
   struct Part {
-    void* dst;
     const void* src;
     size_t bytes;
-  } parts[] = {
-      {p->dev.cols, p->cols.data(), p->cols.size() * sizeof(Column)},
-      {p->dev.table, p->table.data(), p->table.size() * sizeof(double)},
-      {p->dev.slot_ptr, p->slot_ptr.data(), p->slot_ptr.size() * sizeof(int32_t)},
-      {p->dev.slot_idx, p->slot_idx.data(), p->slot_idx.size() * sizeof(int32_t)},
-      {p->dev.mode_col, p->mode_col.data(), p->mode_col.size() * sizeof(int32_t)},
-      {p->dev.mode_N, p->mode_N.data(), p->mode_N.size() * sizeof(int32_t)},
-      {p->dev.split_step, p->split_step.data(), p->split_step.size() * sizeof(uint32_t)},
-      {p->dev.fused_col, p->fused_col.data(), p->fused_col.size() * sizeof(int32_t)},
-      {p->dev.fused_kperm, p->fused_kperm.data(), p->fused_kperm.size() * sizeof(int32_t)},
+  } parts[kPlanSections] = {
+      {p->cols.data(), p->cols.size() * sizeof(Column)},
+      {p->table.data(), p->table.size() * sizeof(double)},
+      {p->slot_ptr.data(), p->slot_ptr.size() * sizeof(int32_t)},
+      {p->slot_idx.data(), p->slot_idx.size() * sizeof(int32_t)},
+      {p->mode_col.data(), p->mode_col.size() * sizeof(int32_t)},
+      {p->mode_N.data(), p->mode_N.size() * sizeof(int32_t)},
+      {p->split_step.data(), p->split_step.size() * sizeof(uint32_t)},
+      {p->fused_col.data(), p->fused_col.size() * sizeof(int32_t)},
+      {p->fused_kperm.data(), p->fused_kperm.size() * sizeof(int32_t)},
   };
-  for (const Part& part : parts) {
-    if (part.bytes == 0) continue;
-    cudaError_t e = async ? cudaMemcpyAsync(part.dst, part.src, part.bytes, cudaMemcpyHostToDevice, stream)
-                          : cudaMemcpy(part.dst, part.src, part.bytes, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_error(e, "copy of plan tables");
-  }
+  // One copy for all sections.
+  const size_t end = off[kPlanSections - 1] + parts[kPlanSections - 1].bytes;
+  std::vector<char> image(end, 0);
+  for (int i = 0; i < kPlanSections; ++i)
+    if (parts[i].bytes) std::memcpy(image.data() + off[i], parts[i].src, parts[i].bytes);
+  if (end == 0) return ZP_OK;
+  const cudaError_t e = async ? cudaMemcpyAsync(base, image.data(), end, cudaMemcpyHostToDevice, stream)
+                              : cudaMemcpy(base, image.data(), end, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return cuda_error(e, "copy of plan tables");
   return ZP_OK;
 }
 
 size_t plan_tri_bytes(const zp_plan* p) { return align_up(p->tri_perm.size() * sizeof(int32_t), 256); }
 
 zp_status plan_tri_upload(zp_plan* p, void* base) {
-  if (!p->tri) return ZP_OK;
+  if (p->tri_perm.empty()) return ZP_OK;
   p->dev.tri_perm = (int32_t*)base;
   const cudaError_t e = cudaMemcpy(base, p->tri_perm.data(), p->tri_perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
   return e == cudaSuccess ? ZP_OK : cuda_error(e, "copy of plan tables");

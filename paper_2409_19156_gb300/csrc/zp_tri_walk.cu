@@ -1,0 +1,265 @@
+// Radial polynomials, rho-derivatives and Z over a whole triangle n <= n_max in float64, by the
+// recursion over neighbouring m (see zp_tri.h for the layout and its derivation):
+//   R_n^m = rho T_0 - R_{n-2}^m,   (R_n^m)^(k) = n T_{k-1} + (R_{n-2}^m)^(k),
+//   T_k = (R_{n-1}^{|m-1|})^(k) + (R_{n-1}^{m+1})^(k)
+// (the derivative form from U_n' = 2n U_{n-1} + U_{n-2}' under the integral).  A value costs 2, 3, 5
+// or 7 float64 operations for k <= 0, 1, 2, 3 against the column recursion's 3, 7, 11 or 15 with its
+// weights, needs no tables, and loses less: an error spreads with weights of at most 1 (radial set
+// n <= 100, k = 0..3: 7e-16 of the norm against 6e-15), while values in the growth region near the
+// origin add terms of one sign and keep their relative accuracy.
+//
+// One warp per 32 points, one point per thread, walking 2 x 2 blocks of (a, b) = ((n+m)/2, (n-m)/2)
+// row by row; the row above (every lane of its derivatives) is kept in shared memory, private to the
+// thread, so nothing synchronises.  Bound: float64 issue (a warp's operation holds its scheduler's
+// pipe for 64 cycles), so a warp per scheduler is enough, and the shared memory may be large; the
+// stores are whole 128-byte lines per warp.  Measured against the column form: radial set n <= 100,
+// k <= 3, 1e5 points 6.32 -> 4.62 ms; Z and dZ/drho with dZ/dtheta, n <= 32, 99991 points 836 -> 631 us.  cos / sin(m theta) come from the fixed-point angle
+// functions on the integer pipe, which is idle here.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "zp_api_common.h"
+#include "zp_internal.h"
+#include "zp_series_internal.h"
+#include "zp_tri.h"
+
+namespace zp {
+namespace {
+
+constexpr int W = 32;  // points per block (one warp)
+
+struct TriWalkArgs {
+  const int32_t* perm;  // modes of every position (zp_tri.h), -1 for none
+  const double* r;
+  const double* theta;
+  int64_t p_end;  // points 0 .. p_end - 1 of P
+  int64_t P, J;
+  double* out;
+  double* out_dtheta;
+  unsigned long long* rowmax;
+  int n_max;
+};
+
+__host__ __device__ constexpr int rows_of(int n_max) { return 2 * (n_max / 4) + 2; }
+__host__ __device__ constexpr uint32_t walk_smem(int n_max, int kmax, bool ang) {
+  return (uint32_t)(rows_of(n_max) * (kmax + 1) * W * 8 + (n_max + 3) * 8 + (ang ? (n_max + 1) * W * 16 : 0));
+}
+
+// v 2^-62 as a float64, rounded to nearest, by integer operations.
+__device__ __forceinline__ double from_fixed62(int64_t v) {
+  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a);
+  const uint64_t m = a << lz;  // top bit set
+  uint64_t b = ((m >> 11) & 0xfffffffffffffull) | ((uint64_t)(1023 - 62 + 63 - lz) << 52);
+  b += (m >> 10) & 1;
+  return __longlong_as_double((long long)(b | ((uint64_t)v & (1ull << 63))));
+}
+
+// cos and sin(m theta), m = 0 .. n_max, of this thread's point.  In fixed point (absolute errors below
+// 2^-57) unless the angle is so small that sin(m theta) needs relative accuracy, or out of its range:
+// then by angle addition in float64, restarted from sincos at every 16th m.
+__device__ __forceinline__ void angle_rows(double th, int n_max, double2* an) {
+  const double mag = fabs(th);
+  if (mag >= 1.0 / 128 && mag < 2048.0) {
+    int64_t ci, si;
+    tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
+    const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
+    TriTrig c = tri_split(1ll << 62), s = tri_split(0);
+    an[0] = make_double2(1.0, 0.0);
+    for (int m = 1; m <= n_max; ++m) {
+      tri_rotate(c, s, c1, s1);
+      an[(size_t)m * W] = make_double2(from_fixed62((int64_t)c.hi * (1ll << 31) + c.lo),
+                                       from_fixed62((int64_t)s.hi * (1ll << 31) + s.lo));
+    }
+  } else {
+    double s1, c1, c = 1.0, s = 0.0;
+    sincos(th, &s1, &c1);
+    for (int m = 0; m <= n_max; ++m) {
+      if (m % 16 == 0) {
+        if (m > 0) sincos((double)m * th, &s, &c);
+      } else {
+        const double cn = fma(c, c1, -s * s1);
+        s = fma(s, c1, c * s1);
+        c = cn;
+      }
+      an[(size_t)m * W] = make_double2(c, s);
+    }
+  }
+}
+
+// KMAX: highest rho-derivative; ANG: Z instead of R; DT (with ANG): also dZ/dtheta.
+template <int KMAX, bool ANG, bool DT>
+__global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
+  extern __shared__ double tri_smem[];
+  constexpr int L = KMAX + 1;
+  const int lane = threadIdx.x, n_max = a.n_max, H = n_max / 2;
+  double2* an = reinterpret_cast<double2*>(tri_smem) + lane;  // [m][lane]
+  double* st = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + lane;  // [b][k][lane]
+  double* num = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)rows_of(n_max) * L * W;  // 0, 1, 2, ..
+  for (int i = lane; i < n_max + 3; i += W) num[i] = (double)i;
+  __syncwarp();
+  const int64_t p = (int64_t)blockIdx.x * W + lane;
+  const bool valid = p < a.p_end;
+  const double rho = valid ? a.r[p] : 0.0;
+  if constexpr (ANG) angle_rows(valid ? a.theta[p] : 0.0, n_max, an);
+  double* const out = a.out + p;
+  double* const out_dt = DT ? a.out_dtheta + p : nullptr;
+  const int64_t order = a.J * a.P;
+
+  auto put = [&](int32_t j, const double (&v)[L], double dt) {
+    if (j < 0) return;
+    double* o = out + (int64_t)j * a.P;
+    if (valid) {
+#pragma unroll
+      for (int k = 0; k < L; ++k) __stcs(o + k * order, v[k]);
+      if constexpr (DT) __stcs(out_dt + (int64_t)j * a.P, dt);
+    }
+    if constexpr (KMAX == 0 && ANG) {
+      if (a.rowmax) {  // the row's largest high word, for the float64-accurate GEMM's scales
+        const uint32_t h = valid ? (uint32_t)__double2hiint(v[0]) & 0x7fffffffu : 0u;
+        const uint32_t mx = __reduce_max_sync(0xffffffffu, h);
+        if (lane == 0) atomicMax(a.rowmax + j, (unsigned long long)mx << 32);
+      }
+    }
+  };
+  auto emit = [&](const double (&f)[L], int32_t jc, int32_t js, int m) {
+    if constexpr (!ANG) {
+      put(jc, f, 0.0);
+      put(js, f, 0.0);
+    } else {
+      if (jc < 0 && js < 0) return;
+      const double2 g = an[(size_t)m * W];
+      double c[L], s[L];
+#pragma unroll
+      for (int k = 0; k < L; ++k) {
+        c[k] = f[k] * g.x;
+        s[k] = f[k] * g.y;
+      }
+      const double md = DT ? num[m] : 0.0;
+      put(jc, c, DT ? -md * s[0] : 0.0);
+      put(js, s, DT ? md * c[0] : 0.0);
+    }
+  };
+
+  const int4* perm = reinterpret_cast<const int4*>(a.perm);
+  int block = 0;
+  for (int A = 0; A <= H; ++A) {
+    const int nb = min(A, H - A);
+    double l0[L], l1[L], dg[L];  // f(2A, 2B-1), f(2A+1, 2B-1), f(2A-1, 2B-1) and their derivatives
+#pragma unroll
+    for (int k = 0; k < L; ++k) l0[k] = l1[k] = dg[k] = 0.0;
+    if (A == 0) dg[0] = -1.0;
+    for (int B = 0; B <= nb; ++B, ++block) {
+      const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
+      double* row = st + (size_t)(2 * B) * L * W;
+      double u0[L], u1[L], e00[L], e01[L], e10[L], e11[L];
+#pragma unroll
+      for (int k = 0; k < L; ++k) {
+        u0[k] = B < A ? row[k * W] : l0[k];
+        u1[k] = B < A ? row[(L + k) * W] : l1[k];
+      }
+      const int n0 = 2 * (A + B), m0 = 2 * (A - B);
+      const double nd0 = num[n0], nd1 = num[n0 + 1], nd2 = num[n0 + 2];
+      // One element from its neighbours above and to the left and the one across.
+      auto element = [&](double (&f)[L], const double (&up)[L], const double (&left)[L], const double (&old)[L], double n) {
+        double t = up[0] + left[0];
+        f[0] = fma(rho, t, -old[0]);
+#pragma unroll
+        for (int k = 1; k < L; ++k) {
+          f[k] = fma(n, t, old[k]);
+          if (k + 1 < L) t = up[k] + left[k];
+        }
+      };
+      element(e00, u0, l0, dg, nd0);
+      element(e01, u1, e00, u0, nd1);
+      element(e10, e00, l1, l0, nd1);
+      element(e11, e01, e10, e00, nd2);
+#pragma unroll
+      for (int k = 0; k < L; ++k) {
+        row[k * W] = e10[k];
+        row[(L + k) * W] = e11[k];
+        dg[k] = u1[k];
+        l0[k] = e01[k];
+        l1[k] = e11[k];
+      }
+      emit(e00, jc.x, js.x, m0);
+      emit(e01, jc.y, js.y, max(m0 - 1, 0));
+      emit(e10, jc.z, js.z, min(m0 + 1, n_max));
+      emit(e11, jc.w, js.w, m0);
+    }
+  }
+}
+
+template <int KMAX, bool ANG, bool DT>
+cudaError_t launch(const TriWalkArgs& a, unsigned blocks, uint32_t smem, cudaStream_t st) {
+  static DeviceMemo<int> memo;
+  int set = 0;
+  const zp_status s = memo.get(&set, [](int* x) -> zp_status {
+    *x = 1;
+    const cudaError_t e = cudaFuncSetAttribute(tri_walk_kernel<KMAX, ANG, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kTriWalkSmem);
+    return e == cudaSuccess ? ZP_OK : cuda_error(e, "triangle walk set-up");
+  });
+  if (s != ZP_OK) return cudaErrorInvalidValue;
+  tri_walk_kernel<KMAX, ANG, DT><<<blocks, W, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int KMAX>
+cudaError_t launch_k(const TriWalkArgs& a, unsigned blocks, uint32_t smem, cudaStream_t st) {
+  if (a.theta == nullptr) return launch<KMAX, false, false>(a, blocks, smem, st);
+  return a.out_dtheta ? launch<KMAX, true, true>(a, blocks, smem, st) : launch<KMAX, true, false>(a, blocks, smem, st);
+}
+
+}  // namespace
+
+int64_t tri_walk_points(const zp_plan* plan, int64_t n_points, int max_deriv, bool ang, bool dtheta, int sms) {
+  if (!plan->dev.tri_perm || walk_smem(plan->n_max, max_deriv, ang) > kTriWalkSmem) return 0;
+  // Float64 operations per point of either form.
+  const int64_t pairs = (int64_t)(plan->n_max / 2 + 1) * ((plan->n_max + 1) / 2 + 1);
+  const int64_t per_value = max_deriv == 0 ? 2 : 2 * max_deriv + 1;
+  const int64_t out_ops = ang ? plan->n_modes * (max_deriv + 1 + (dtheta ? 1 : 0)) : 0;
+  int64_t steps = 0;
+  for (const Column& c : plan->cols) steps += c.n_steps;
+  const int64_t tri = pairs * per_value + out_ops, col = steps * (4 * max_deriv + 3) + out_ops;
+  // The walk runs a warp per scheduler in whole waves of 4 sms warps; what is left over takes the
+  // column form, which spreads a point over its columns.  An operation costs the walk about 4/3 of
+  // the column form's time (its float64 pipe waits for shared memory and stores where the column
+  // form's eight steps overlap: radial set n <= 100, k <= 3: 440 against 622 G operations/s).
+  const int64_t wave = 4 * (int64_t)sms * W;
+  int64_t points = n_points / wave * wave;
+  const int64_t rest = n_points - points;
+  if (3 * rest * col > 4 * wave * tri) points = n_points;
+  return 4 * tri < 3 * col ? points : 0;
+}
+
+zp_status launch_tri_walk(const zp_plan* plan, const double* r, const double* theta, int64_t n_points, int64_t p_end,
+                          int max_deriv, double* out, double* out_dtheta, unsigned long long* rowmax, cudaStream_t stream) {
+  TriWalkArgs a;
+  a.perm = plan->dev.tri_perm;
+  a.r = r;
+  a.theta = theta;
+  a.p_end = p_end;
+  a.P = n_points;
+  a.J = plan->n_modes;
+  a.out = out;
+  a.out_dtheta = out_dtheta;
+  a.rowmax = rowmax;
+  a.n_max = plan->n_max;
+  const int64_t blocks = (p_end + W - 1) / W;
+  if (blocks > 0x7fffffffLL) return set_error(ZP_ERR_INVALID_ARG, "n_points too large for one launch");
+  const uint32_t smem = walk_smem(plan->n_max, max_deriv, theta != nullptr);
+  cudaError_t e;
+  switch (max_deriv) {
+    case 0: e = launch_k<0>(a, (unsigned)blocks, smem, stream); break;
+    case 1: e = launch_k<1>(a, (unsigned)blocks, smem, stream); break;
+    case 2: e = launch_k<2>(a, (unsigned)blocks, smem, stream); break;
+    default: e = launch_k<3>(a, (unsigned)blocks, smem, stream); break;
+  }
+  return e == cudaSuccess ? ZP_OK : cuda_error(e, "tri_walk_kernel launch");
+}
+
+}  // namespace zp

@@ -45,6 +45,7 @@ struct WalkArgs {
   const double* theta;
   int64_t P;
   int64_t J;
+  int64_t p_first = 0;  // the launch's first point
   double* out;
   double* out_dtheta;
   // Optional point tables [j][P] (NULL: computed per thread): pw = rho^j (j <= pw_max),
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(TPB) walk_kernel(WalkArgs a) {
   }
   __syncthreads();
 
-  const int64_t p0 = ((int64_t)blockIdx.x * TPB + (int64_t)threadIdx.x) * PPT;
+  const int64_t p0 = a.p_first + ((int64_t)blockIdx.x * TPB + (int64_t)threadIdx.x) * PPT;
   if (p0 >= a.P) return;
   const bool two = PPT == 2 && p0 + 1 < a.P;
   const int m = col.m;
@@ -433,9 +434,20 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t n_cols = (int64_t)plan->cols.size();
-  const bool small = ((n_points + kThreads * kPPT - 1) / (kThreads * kPPT)) * n_cols < 8 * (int64_t)sms;
+  // Mode lists that fill their triangle take the walk over neighbouring m for the points that make
+  // whole waves of it.
+  a.p_first = tri_walk_points(plan, n_points, max_deriv, theta != nullptr, out_dtheta != nullptr, sms);
+  if (a.p_first > 0) {
+    ZP_TRY(launch_tri_walk(plan, r, theta, n_points, a.p_first, max_deriv, out, out_dtheta, rowmax, stream));
+    if (a.p_first == n_points) {
+      timer.mark(2);
+      return timer.finish();
+    }
+  }
+  const int64_t n_left = n_points - a.p_first;
+  const bool small = ((n_left + kThreads * kPPT - 1) / (kThreads * kPPT)) * n_cols < 8 * (int64_t)sms;
   const int64_t per_block = small ? kThreadsSmall : kThreads * kPPT;
-  const int64_t blocks_x = (n_points + per_block - 1) / per_block;
+  const int64_t blocks_x = (n_left + per_block - 1) / per_block;
   if (blocks_x > 0x7fffffffLL) return set_error(ZP_ERR_INVALID_ARG, "n_points too large for one launch");
   dim3 grid((unsigned)blocks_x, (unsigned)n_cols);
   const size_t smem = (size_t)(kHeaderRows + plan->max_steps) * kRow * sizeof(double) +
@@ -449,7 +461,7 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
   int m_max = 0;
   for (const Column& c : plan->cols) m_max = std::max(m_max, (int)c.m);
   ScratchBuffer tables;
-  if (n_points >= 8192 && plan->cols.size() >= 4 && m_max <= 128) {
+  if (n_left >= 8192 && a.p_first == 0 && plan->cols.size() >= 4 && m_max <= 128) {
     const int pw_max = m_max + 2;
     const size_t rows = (size_t)(pw_max + 1) + (ang ? 2 * (size_t)(m_max + 1) : 0);
     // The tables are an optimisation: without the memory for them the walk computes its seeds.
