@@ -122,7 +122,9 @@ def check(fn: str, status: int) -> None:
 
 
 def call(fn: str, *args) -> None:
-    check(fn, getattr(load(), fn)(*args))
+    status = getattr(_lib or load(), fn)(*args)
+    if status != 0:
+        check(fn, status)
 
 
 def modes_i32(x) -> np.ndarray:
@@ -132,8 +134,15 @@ def modes_i32(x) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(x, dtype=np.int64).astype(np.int32))
 
 
+def modes_view(x) -> np.ndarray:
+    """A mode list for the duration of one call: an int32 array as it is, anything else copied."""
+    if type(x) is np.ndarray and x.dtype == np.int32 and x.flags.c_contiguous:
+        return x
+    return modes_i32(x)
+
+
 def i32_ptr(a: np.ndarray):
-    return a.ctypes.data_as(c_i32p)
+    return ctypes.cast(a.__array_interface__["data"][0], c_i32p)
 
 
 class ZpInstance(ctypes.Structure):

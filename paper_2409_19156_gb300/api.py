@@ -24,12 +24,25 @@ from . import _lib
 PREC = {"fp64": 0, "bf16x3": 1, "tf32": 2, "fp64emu": 4}
 
 
-def _stream(device: torch.device) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+# The stream pointer without building a torch.cuda.Stream (2 us of a small call's 16 us of host time).
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
+def _stream(device: torch.device) -> int:
+    return _raw_stream(torch.cuda.current_device() if device.index is None else device.index)
+
+
+def _call(device: torch.device, fn: str, *args) -> None:
+    """One entry point on `device`, switching to it only when it is not the current one."""
+    if device.index is None or device.index == torch.cuda.current_device():
+        _lib.call(fn, *args)
+    else:
+        with torch.cuda.device(device):
+            _lib.call(fn, *args)
 
 
 def _dev_f64(t: torch.Tensor, name: str) -> torch.Tensor:
-    if not isinstance(t, torch.Tensor) or t.device.type != "cuda":
+    if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != torch.float64:
         raise TypeError(f"{name} must be float64")
@@ -74,17 +87,16 @@ class Plan:
 
 def radial(n, m, r: torch.Tensor, max_deriv: int = 0, plan: Plan | None = None, out=None) -> torch.Tensor:
     r = _dev_f64(r, "r")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P = len(nn), r.numel()
     if out is None:
-        out = torch.empty((max_deriv + 1, J, P), dtype=torch.float64, device=r.device)
+        out = r.new_empty((max_deriv + 1, J, P))
     st = _stream(r.device)
-    with torch.cuda.device(r.device):
-        if plan is not None:
-            _lib.call("zp_radial_plan", plan.handle, r.data_ptr(), P, max_deriv, out.data_ptr(), st)
-        else:
-            _lib.call("zp_radial", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), P, max_deriv,
-                      out.data_ptr(), st)
+    if plan is not None:
+        _call(r.device, "zp_radial_plan", plan.handle, r.data_ptr(), P, max_deriv, out.data_ptr(), st)
+    else:
+        _call(r.device, "zp_radial", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), P, max_deriv,
+              out.data_ptr(), st)
     return out
 
 
@@ -94,26 +106,24 @@ def basis(n, m, r: torch.Tensor, theta: torch.Tensor, max_deriv: int = 0, dtheta
     theta = _dev_f64(theta, "theta")
     if theta.numel() != r.numel():
         raise ValueError("r and theta must have the same length")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P = len(nn), r.numel()
-    out = torch.empty((max_deriv + 1, J, P), dtype=torch.float64, device=r.device)
-    dt = torch.empty((J, P), dtype=torch.float64, device=r.device) if dtheta else None
+    out = r.new_empty((max_deriv + 1, J, P))
+    dt = r.new_empty((J, P)) if dtheta else None
     st = _stream(r.device)
-    with torch.cuda.device(r.device):
-        if plan is not None:
-            _lib.call("zp_basis_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P, max_deriv, out.data_ptr(),
-                      _lib.ptr(dt), st)
-        else:
-            _lib.call("zp_basis", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P, max_deriv,
-                      out.data_ptr(), _lib.ptr(dt), st)
+    if plan is not None:
+        _call(r.device, "zp_basis_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P, max_deriv, out.data_ptr(),
+              _lib.ptr(dt), st)
+    else:
+        _call(r.device, "zp_basis", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P, max_deriv,
+              out.data_ptr(), _lib.ptr(dt), st)
     return out, dt
 
 
 def radial_per_mode(plan: Plan, r: torch.Tensor) -> torch.Tensor:
     r = _dev_f64(r, "r")
-    out = torch.empty((plan.n_modes, r.numel()), dtype=torch.float64, device=r.device)
-    with torch.cuda.device(r.device):
-        _lib.call("zp_radial_per_mode", plan.handle, r.data_ptr(), r.numel(), out.data_ptr(), _stream(r.device))
+    out = r.new_empty((plan.n_modes, r.numel()))
+    _call(r.device, "zp_radial_per_mode", plan.handle, r.data_ptr(), r.numel(), out.data_ptr(), _stream(r.device))
     return out
 
 
@@ -121,21 +131,20 @@ def series_eval(n, m, r, theta, coeffs, prec: str = "fp64emu", plan: Plan | None
     r = _dev_f64(r, "r")
     theta = _dev_f64(theta, "theta")
     coeffs = _dev_f64(coeffs, "coeffs")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P = len(nn), r.numel()
     if coeffs.dim() != 2 or coeffs.shape[0] != J:
         raise ValueError("coeffs must be [n_modes, n_sets]")
     S = coeffs.shape[1]
     dtype = torch.float64 if prec in ("fp64", "fp64emu") else torch.float32
-    out = torch.empty((P, S), dtype=dtype, device=r.device)
+    out = r.new_empty((P, S), dtype=dtype)
     st = _stream(r.device)
-    with torch.cuda.device(r.device):
-        if plan is not None:
-            _lib.call("zp_series_eval_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(), S,
-                      PREC[prec], out.data_ptr(), st)
-        else:
-            _lib.call("zp_series_eval", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P,
-                      coeffs.data_ptr(), S, PREC[prec], out.data_ptr(), st)
+    if plan is not None:
+        _call(r.device, "zp_series_eval_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(), S,
+              PREC[prec], out.data_ptr(), st)
+    else:
+        _call(r.device, "zp_series_eval", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P,
+              coeffs.data_ptr(), S, PREC[prec], out.data_ptr(), st)
     return out
 
 
@@ -150,7 +159,7 @@ def series_adjoint(n, m, r, theta, coeffs, grad_out, need=(True, True, True), pl
     theta = _dev_f64(theta, "theta")
     coeffs = _dev_f64(coeffs, "coeffs")
     grad_out = _dev_f64(grad_out, "grad_out")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P = len(nn), r.numel()
     S = coeffs.shape[1]
     if grad_out.shape != (P, S):
@@ -160,14 +169,13 @@ def series_adjoint(n, m, r, theta, coeffs, grad_out, need=(True, True, True), pl
     gr = torch.empty(P, dtype=torch.float64, device=dev) if need[1] else None
     gt = torch.empty(P, dtype=torch.float64, device=dev) if need[2] else None
     st = _stream(dev)
-    with torch.cuda.device(dev):
-        if plan is None and prec == "fp64emu":
-            _lib.call("zp_series_adjoint", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P,
-                      coeffs.data_ptr(), S, grad_out.data_ptr(), _lib.ptr(gC), _lib.ptr(gr), _lib.ptr(gt), st)
-        else:
-            pl = plan if plan is not None else Plan(nn, mm, device=dev)
-            _lib.call("zp_series_adjoint_plan_prec", pl.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(),
-                      S, grad_out.data_ptr(), _lib.ptr(gC), _lib.ptr(gr), _lib.ptr(gt), PREC[prec], st)
+    if plan is None and prec == "fp64emu":
+        _call(dev, "zp_series_adjoint", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(), P,
+              coeffs.data_ptr(), S, grad_out.data_ptr(), _lib.ptr(gC), _lib.ptr(gr), _lib.ptr(gt), st)
+    else:
+        pl = plan if plan is not None else Plan(nn, mm, device=dev)
+        _call(dev, "zp_series_adjoint_plan_prec", pl.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(),
+              S, grad_out.data_ptr(), _lib.ptr(gC), _lib.ptr(gr), _lib.ptr(gt), PREC[prec], st)
     return gC, gr, gt
 
 
@@ -178,20 +186,19 @@ def series_point_hessian(n, m, r, theta, coeffs, grad_out, plan: Plan | None = N
     theta = _dev_f64(theta, "theta")
     coeffs = _dev_f64(coeffs, "coeffs")
     G = _dev_f64(grad_out, "grad_out")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P, S = len(nn), r.numel(), coeffs.shape[1]
     if G.shape != (P, S):
         raise ValueError("grad_out must be [n_points, n_sets]")
     outs = [torch.empty(P, dtype=torch.float64, device=r.device) for _ in range(5)]
     ptrs = [o.data_ptr() for o in outs]
     st = _stream(r.device)
-    with torch.cuda.device(r.device):
-        if plan is not None:
-            _lib.call("zp_series_point_hessian_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(),
-                      S, G.data_ptr(), *ptrs, st)
-        else:
-            _lib.call("zp_series_point_hessian", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(),
-                      P, coeffs.data_ptr(), S, G.data_ptr(), *ptrs, st)
+    if plan is not None:
+        _call(r.device, "zp_series_point_hessian_plan", plan.handle, r.data_ptr(), theta.data_ptr(), P,
+              coeffs.data_ptr(), S, G.data_ptr(), *ptrs, st)
+    else:
+        _call(r.device, "zp_series_point_hessian", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(),
+              theta.data_ptr(), P, coeffs.data_ptr(), S, G.data_ptr(), *ptrs, st)
     return tuple(outs)
 
 
@@ -211,10 +218,9 @@ def series_point_hvp(n, m, r, theta, coeffs, grad_out, v_r, v_theta, plan: Plan 
     pl = plan if plan is not None else Plan(n, m, device=r.device)
     hv_r = torch.empty(P, dtype=torch.float64, device=r.device)
     hv_t = torch.empty(P, dtype=torch.float64, device=r.device)
-    with torch.cuda.device(r.device):
-        _lib.call("zp_series_point_hvp_plan", pl.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(), S,
-                  G.data_ptr(), v_r.data_ptr(), v_theta.data_ptr(), hv_r.data_ptr(), hv_t.data_ptr(),
-                  _stream(r.device))
+    _call(r.device, "zp_series_point_hvp_plan", pl.handle, r.data_ptr(), theta.data_ptr(), P, coeffs.data_ptr(), S,
+          G.data_ptr(), v_r.data_ptr(), v_theta.data_ptr(), hv_r.data_ptr(), hv_t.data_ptr(),
+          _stream(r.device))
     return hv_r, hv_t
 
 
@@ -229,21 +235,20 @@ def series_fit(n, m, r, theta, samples, weights=None, ridge: float = 0.0, plan: 
     theta = _dev_f64(theta, "theta")
     Y = _dev_f64(samples, "samples")
     w = None if weights is None else _dev_f64(weights, "weights")
-    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_i32(n), _lib.modes_i32(m))
+    nn, mm = (plan.n, plan.m) if plan is not None else (_lib.modes_view(n), _lib.modes_view(m))
     J, P = len(nn), r.numel()
     if Y.dim() != 2 or Y.shape[0] != P:
         raise ValueError("samples must be [n_points, n_sets]")
     S = Y.shape[1]
     out = torch.empty((J, S), dtype=torch.float64, device=r.device)
     st = _stream(r.device)
-    with torch.cuda.device(r.device):
-        if plan is None and prec == "fp64emu":
-            _lib.call("zp_series_fit", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(),
-                      _lib.ptr(w), P, Y.data_ptr(), S, float(ridge), out.data_ptr(), st)
-        else:
-            pl = plan if plan is not None else Plan(nn, mm, device=r.device)
-            _lib.call("zp_series_fit_plan_prec", pl.handle, r.data_ptr(), theta.data_ptr(), _lib.ptr(w), P,
-                      Y.data_ptr(), S, float(ridge), out.data_ptr(), PREC[prec], st)
+    if plan is None and prec == "fp64emu":
+        _call(r.device, "zp_series_fit", _lib.i32_ptr(nn), _lib.i32_ptr(mm), J, r.data_ptr(), theta.data_ptr(),
+              _lib.ptr(w), P, Y.data_ptr(), S, float(ridge), out.data_ptr(), st)
+    else:
+        pl = plan if plan is not None else Plan(nn, mm, device=r.device)
+        _call(r.device, "zp_series_fit_plan_prec", pl.handle, r.data_ptr(), theta.data_ptr(), _lib.ptr(w), P,
+              Y.data_ptr(), S, float(ridge), out.data_ptr(), PREC[prec], st)
     return out
 
 
