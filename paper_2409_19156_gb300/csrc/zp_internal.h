@@ -73,7 +73,8 @@ struct DevicePlanTables {
   int32_t* mode_col = nullptr;  // [n_modes]: column index of every mode
   int32_t* mode_N = nullptr;    // [n_modes]: Jacobi degree of every mode
   uint2* split_step = nullptr;  // [table rows]: step descriptors of the split basis
-  int32_t* tri_perm = nullptr;  // [tri_chunks * 16]: mode of every triangle position, -1 for none; NULL without the layout
+  int32_t* tri_perm = nullptr;  // [tri_chunks * 16]: mode of every triangle position, -1 for none; NULL without the layout;
+                                // followed by tri_order
   int4* fused_col = nullptr;    // [columns]: fused contraction layout (see kFusedKind*)
   int32_t* fused_kperm = nullptr;  // [fused_kpad]: slot of every K position, -1 for padding
 };
@@ -98,6 +99,8 @@ struct zp_plan {
   int32_t fused_ep = 1;              // row scale exponent of the fused kernel on the unit disc
   bool tri = false;                  // the fused series takes the triangle layout (zp_tri.h)
   std::vector<int32_t> tri_perm;     // the layout's positions' modes (empty without it)
+  std::vector<int32_t> tri_order;    // modes in the split basis's K order: whole blocks, then the others
+  int32_t tri_full = 0;              // whole blocks: all of their eight positions have modes
   zp::DevicePlanTables dev;
   size_t device_bytes = 0;
   void* dev_block = nullptr;  // single allocation backing dev.*
@@ -121,10 +124,10 @@ size_t plan_device_layout(const zp_plan* p, size_t offsets[kPlanSections]);
 // Points p->dev at `base` (laid out as plan_device_layout) and copies the host tables there,
 // with cudaMemcpyAsync on `stream` when async, else synchronously.
 zp_status plan_upload(zp_plan* p, void* base, cudaStream_t stream, bool async);
-// The triangle layout's table, kept behind that block by plans that own their device memory: its
-// size in bytes (a multiple of 256, 0 without the layout) and its upload (synchronous).
+// The triangle layout's tables, kept behind that block: their size in bytes (a multiple of 256, 0
+// without the layout) and their upload, as above.
 size_t plan_tri_bytes(const zp_plan* p);
-zp_status plan_tri_upload(zp_plan* p, void* base);
+zp_status plan_tri_upload(zp_plan* p, void* base, cudaStream_t stream = nullptr, bool async = false);
 // Cached plan for a mode list on the current device (created on first use).  The caller
 // keeps *out alive while it uses the plan; the cache may drop its own reference.
 zp_status cached_plan(const int32_t* n, const int32_t* m, int64_t n_modes, std::shared_ptr<const zp_plan>* out);

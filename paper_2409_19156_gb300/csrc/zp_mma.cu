@@ -346,6 +346,172 @@ __device__ __forceinline__ void split_basis_tile(const BasisArgs& a, int64_t til
   while (k % C::BK != 0) push1(zeros);
 }
 
+// ---------------------------------------------------------------------------------------
+// The same operand from the fixed-point triangle walk (zp_tri.h), for mode lists that have its
+// layout.  The float64 recursion above holds the float64 pipe for two operations per (n, |m|) and
+// point; here the walk runs on the integer pipe in 64-bit fixed point, the values become float32
+// from their upper 32 bits (2^-31 absolute; the operands keep 16 or 11 significant bits of their
+// own) and the angular products stay float32.  K order: first the blocks whose eight elements
+// (four cos, four sin) all have modes, eight positions each, so that a block is a whole 16-byte unit
+// per operand part with no packing across blocks; then the other blocks' modes one by one.
+struct TriBasisArgs {
+  const int32_t* perm;  // modes of the triangle's positions, -1 for none
+  const double* r;
+  const double* theta;
+  int64_t P;
+  int64_t mt_base;
+  int KC;
+  uint8_t* A;
+  int n_max;
+  int full;  // blocks with all modes
+};
+
+__host__ __device__ constexpr uint32_t tri_basis_smem(int n_max) {
+  return (uint32_t)((2 * (n_max / 4) + 2) * BM * 8 + (n_max + 1) * BM * 8);
+}
+// Two blocks or more per SM.
+constexpr uint32_t kTriBasisSmem = 110 * 1024;
+
+template <bool TF32, bool SLOW>
+__device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA, uint32_t row, double rho, double th,
+                                              uint64_t* st, float2* an) {
+  using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
+  constexpr int UNIT = TF32 ? 4 : 8;
+  const int n_max = a.n_max, H = n_max / 2;
+  TriPoint tp = {};
+  if constexpr (!SLOW) {
+    tp = tri_point((uint64_t)__double_as_longlong(rho));
+    int64_t ci, si;
+    tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
+    const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
+    TriTrig c = tri_split(1ll << 62), s = tri_split(0);
+    for (int m = 0; m <= n_max; ++m) {
+      // 2^-31 of the angle's word, 2^-30 of the radial one.
+      an[(size_t)m * BM] = make_float2((float)c.hi * 0x1p-61f, (float)s.hi * 0x1p-61f);
+      tri_rotate(c, s, c1, s1);
+    }
+  } else {
+    double s1, c1, c = 1.0, s = 0.0;
+    sincos(th, &s1, &c1);
+    for (int m = 0; m <= n_max; ++m) {
+      an[(size_t)m * BM] = make_float2(float_of_double(c), float_of_double(s));
+      const double cn = fma(c, c1, -s * s1);
+      s = fma(s, c1, c * s1);
+      c = cn;
+    }
+  }
+  int k_full = 0, k_tail = 8 * a.full;
+  Pack16 hi, lo;
+  auto at = [&](int k) {  // byte offset of a unit's first position
+    uint8_t* chunk = gA + (size_t)(k / C::BK) * C::A_CHUNK;
+    if constexpr (TF32) return chunk + ptx::sw_offset_b32<C::ROW>(row, (uint32_t)(k % C::BK));
+    else return chunk + ptx::sw_offset_b16<C::ROW>(row, (uint32_t)(k % C::BK));
+  };
+  auto tail = [&](float z) {
+    if constexpr (TF32) {
+      hi.push32(__float_as_uint(to_tf32(z)));
+    } else {
+      const uint32_t h = bf16x2_bits(z, 0.0f) & 0xffffu;
+      hi.push16(h);
+      lo.push16(bf16x2_bits(z - __uint_as_float(h << 16), 0.0f) & 0xffffu);
+    }
+    if (++k_tail % UNIT == 0) {
+      uint8_t* dst = at(k_tail - UNIT);
+      hi.store(dst);
+      if constexpr (!TF32) lo.store(dst + C::A_PART);
+    }
+  };
+  const int4* perm = reinterpret_cast<const int4*>(a.perm);
+  int block = 0;
+  for (int A = 0; A <= H; ++A) {
+    const int nb = min(A, H - A);
+    uint64_t l0 = SLOW ? 0ull : kTriZero, l1 = l0;
+    uint64_t dg = A == 0 ? (SLOW ? (uint64_t)__double_as_longlong(-1.0) : 0ull) : l0;
+    for (int B = 0; B <= nb; ++B, ++block) {
+      const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
+      uint64_t* sr = st + (size_t)(2 * B) * BM;
+      const uint64_t u0 = B < A ? sr[0] : l0, u1 = B < A ? sr[BM] : l1;
+      uint64_t e00, e01, e10, e11;
+      float f[4];
+      if constexpr (!SLOW) {
+        e00 = tri_step(tp, u0, l0, dg);
+        e01 = tri_step(tp, u1, e00, u0);
+        e10 = tri_step(tp, e00, l1, l0);
+        e11 = tri_step(tp, e01, e10, e00);
+        auto upper = [](uint64_t e) { return (float)(int32_t)((uint32_t)(e >> 31) - (1u << 30)); };
+        f[0] = upper(e00);
+        f[1] = upper(e01);
+        f[2] = upper(e10);
+        f[3] = upper(e11);
+      } else {
+        auto d = [](uint64_t v) { return __longlong_as_double((long long)v); };
+        auto w = [](double v) { return (uint64_t)__double_as_longlong(v); };
+        const double x00 = fma(rho, d(u0) + d(l0), -d(dg)), x01 = fma(rho, d(u1) + x00, -d(u0));
+        const double x10 = fma(rho, x00 + d(l1), -d(l0)), x11 = fma(rho, x01 + x10, -x00);
+        e00 = w(x00);
+        e01 = w(x01);
+        e10 = w(x10);
+        e11 = w(x11);
+        f[0] = float_of_double(x00);
+        f[1] = float_of_double(x01);
+        f[2] = float_of_double(x10);
+        f[3] = float_of_double(x11);
+      }
+      sr[0] = e10;
+      sr[BM] = e11;
+      dg = u1;
+      l0 = e01;
+      l1 = e11;
+      const int m0 = 2 * (A - B);
+      const float2 mid = an[(size_t)m0 * BM], low = an[(size_t)max(m0 - 1, 0) * BM], top = an[(size_t)min(m0 + 1, n_max) * BM];
+      const float z[8] = {f[0] * mid.x, f[1] * low.x, f[2] * top.x, f[3] * mid.x,
+                          f[0] * mid.y, f[1] * low.y, f[2] * top.y, f[3] * mid.y};
+      if ((jc.x | jc.y | jc.z | jc.w | js.x | js.y | js.z | js.w) >= 0) {
+        if constexpr (TF32) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            *reinterpret_cast<float4*>(at(k_full + 4 * i)) =
+                make_float4(to_tf32(z[4 * i]), to_tf32(z[4 * i + 1]), to_tf32(z[4 * i + 2]), to_tf32(z[4 * i + 3]));
+        } else {
+          uint32_t h[4], l[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            h[i] = bf16x2_bits(z[2 * i], z[2 * i + 1]);
+            l[i] = bf16x2_bits(z[2 * i] - __uint_as_float(h[i] << 16), z[2 * i + 1] - __uint_as_float(h[i] & 0xffff0000u));
+          }
+          uint8_t* dst = at(k_full);
+          *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+          *reinterpret_cast<uint4*>(dst + C::A_PART) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+        k_full += 8;
+      } else {
+        const int32_t j[8] = {jc.x, jc.y, jc.z, jc.w, js.x, js.y, js.z, js.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (j[i] >= 0) tail(z[i]);
+      }
+    }
+  }
+  while (k_tail % C::BK != 0) tail(0.0f);
+}
+
+template <bool TF32>
+__global__ void __launch_bounds__(BM) tri_basis_kernel(TriBasisArgs a) {
+  using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
+  extern __shared__ uint64_t tri_basis_mem[];
+  uint64_t* st = tri_basis_mem + threadIdx.x;
+  float2* an = reinterpret_cast<float2*>(tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM) + threadIdx.x;
+  const int64_t p = (a.mt_base + blockIdx.x) * BM + threadIdx.x;
+  const bool valid = p < a.P;
+  const double rho = valid ? a.r[p] : 0.0, th = valid ? a.theta[p] : 0.0;
+  const uint32_t e = ((uint32_t)__double2hiint(th) >> 20) & 0x7ffu;
+  uint8_t* gA = a.A + (size_t)blockIdx.x * a.KC * C::A_CHUNK;
+  if (__any_sync(0xffffffffu, !(rho >= 0.0 && rho <= 1.0 && e < (uint32_t)kTriAngleExponent)))
+    tri_basis_row<TF32, true>(a, gA, threadIdx.x, rho, th, st, an);
+  else
+    tri_basis_row<TF32, false>(a, gA, threadIdx.x, rho, th, st, an);
+}
+
 struct CoeffArgs {
   const double* coeffs;  // [J][S]
   const int32_t* slot_idx;
@@ -1184,10 +1350,16 @@ zp_status run_split(const zp_plan* plan, const double* r, const double* theta, i
       *x = 1;
     }
     // The coefficient kernel's shared memory limit, set once per device.
-    const cudaError_t e = cudaFuncSetAttribute(split_coeff_kernel<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>::B_CHUNK + 1024));
+    cudaError_t e = cudaFuncSetAttribute(split_coeff_kernel<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>::B_CHUNK + 1024));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(tri_basis_kernel<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriBasisSmem);
     return e == cudaSuccess ? ZP_OK : cuda_error(e, "cudaFuncSetAttribute(split_coeff_kernel)");
   }));
+  // The basis from the triangle walk where the mode list has its layout and a tile's state fits.
+  const uint32_t tri_smem = tri_basis_smem(plan->n_max);
+  const bool tri = plan->dev.tri_perm && tri_smem <= kTriBasisSmem;
+  if (tri) per_sm = (int)std::min<uint32_t>(8, 232448u / (tri_smem + 1024));
   const int64_t wave = (int64_t)std::max(per_sm, 1) * gs.sms;
   int64_t slab = 0;
   if (preset) {
@@ -1217,7 +1389,7 @@ zp_status run_split(const zp_plan* plan, const double* r, const double* theta, i
   const uint32_t coeff_smem = C::B_CHUNK + 1024;
   cudaError_t e;
 
-  CoeffArgs ca{coeffs, plan->dev.slot_idx, J, S, KC, B};
+  CoeffArgs ca{coeffs, tri ? plan->dev.tri_perm + plan->tri_perm.size() : plan->dev.slot_idx, J, S, KC, B};
   timer.begin(0, &ev0, stream);
   split_coeff_kernel<TF32><<<(unsigned)(NT * KC), kCoeffThreads, coeff_smem, stream>>>(ca);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "split_coeff_kernel launch");
@@ -1229,7 +1401,12 @@ zp_status run_split(const zp_plan* plan, const double* r, const double* theta, i
                  plan->dev.slot_idx,
                  r, theta, P, mt0, KC, A};
     timer.begin(1, &ev0, stream);
-    split_basis_kernel<TF32><<<(unsigned)tiles, basis_threads<TF32>(), 0, stream>>>(ba, tiles);
+    if (tri) {
+      const TriBasisArgs ta{plan->dev.tri_perm, r, theta, P, mt0, KC, A, plan->n_max, plan->tri_full};
+      tri_basis_kernel<TF32><<<(unsigned)tiles, BM, tri_smem, stream>>>(ta);
+    } else {
+      split_basis_kernel<TF32><<<(unsigned)tiles, basis_threads<TF32>(), 0, stream>>>(ba, tiles);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "split_basis_kernel launch");
     timer.end(1, ev0, stream);
     GemmArgs ga{A, B, out, P, S, mt0, tiles, NT, KC};

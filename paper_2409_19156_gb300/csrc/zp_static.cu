@@ -98,7 +98,7 @@ static zp_status zp_series_eval_static_impl(const int32_t* n, const int32_t* m, 
   }
   // Layout of the static array: plan tables | coefficient tiles | basis slab.
   size_t offsets[kPlanSections];
-  const size_t table_bytes = round_up(plan_device_layout(&plan, offsets), 1024);
+  size_t table_bytes = round_up(plan_device_layout(&plan, offsets), 1024);
   size_t b_bytes = 0, tile_bytes = 0;
   const size_t need = table_bytes + round_up(split_scratch_bytes(prec, n_modes, n_sets, &b_bytes, &tile_bytes), 1024);
   if (need > (size_t)ZP_STATIC_SCRATCH_BYTES) {
@@ -107,12 +107,17 @@ static zp_status zp_series_eval_static_impl(const int32_t* n, const int32_t* m, 
                      "and one 128-point basis tile) but ZP_STATIC_SCRATCH_BYTES is " +
                          std::to_string((size_t)ZP_STATIC_SCRATCH_BYTES) + "; use zp_series_eval instead");
   }
+  // The triangle layout's tables too, where there is room (else the walk by columns).
+  const size_t tri_at = table_bytes, tri_bytes = round_up(plan_tri_bytes(&plan), 1024);
+  const bool tri = tri_bytes > 0 && need + tri_bytes <= (size_t)ZP_STATIC_SCRATCH_BYTES;
+  if (tri) table_bytes += tri_bytes;
   void* base = nullptr;
   ZP_TRY(static_scratch_address(&base));
   unsigned char* bytes = (unsigned char*)base;
   // Tables: pageable host -> device copies on the caller's stream (ordered after any
   // earlier call on that stream, which may still be reading the previous tables).
   ZP_TRY(plan_upload(&plan, bytes, st, true));
+  if (tri) ZP_TRY(plan_tri_upload(&plan, bytes + tri_at, st, true));
   SplitScratch sc;
   sc.b = bytes + table_bytes;
   sc.b_bytes = round_up(b_bytes, 1024);

@@ -119,3 +119,26 @@ def test_float64_walk_against_oracle(n_max, k, which):
         assert (np.abs(dt - np.array(wt)) <= 1e-11 * np.maximum(ns, 1)[:, None] * 1.02 ** ns[:, None]).all()
     far = np.where(r[rows] > 1.0, 8.0 ** np.minimum(n_max, 12), 1.0)  # values beyond the rim grow past 1
     assert (np.abs(got - np.array(want)) <= tol * far).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec,bound", [("bf16x3", 1e-4), ("tf32", 2e-3)])
+@pytest.mark.parametrize("n_max,P,S,which", [(0, 1, 1, "full"), (1, 130, 3, "full"), (7, 127, 5, "most"), (32, 700, 20, "full"),
+                                             (45, 300, 257, "most"), (64, 129, 4, "full"), (70, 129, 4, "full")])
+def test_split_series_against_the_baseline(n_max, P, S, which, prec, bound):
+    """Split-precision series on both sides of the triangle basis's largest degree, with whole and
+    part-filled blocks: the bounds of the other split tests, relative to the sums of magnitudes."""
+    torch = pytest.importorskip("torch")
+    import paper_2409_19156_gb300 as zp
+
+    ns, ms = _lists(n_max, which)
+    r, th = inputs.sqrt_uniform_points(P, 5 + n_max)
+    if P > 500:
+        r[300:303], th[303] = [1.0, 1.02, 0.0], -7.0
+    C = inputs.scaled_normal_coeffs(ns, S, n_max)
+    r, th, C = (torch.as_tensor(x, device="cuda") for x in (r, th, C))
+    plan = zp.Plan(ns, ms)
+    got = zp.series_eval(None, None, r, th, C, prec=prec, plan=plan).double()
+    want = zp.series_eval(None, None, r, th, C, prec="fp64", plan=plan)
+    size = zp.basis(None, None, r, th, 0, plan=plan)[0][0].abs().T @ C.abs()
+    assert bool(((got - want).abs() <= bound * size + 1e-6).all())
