@@ -367,28 +367,39 @@ struct TriBasisArgs {
 };
 
 __host__ __device__ constexpr uint32_t tri_basis_smem(int n_max) {
-  return (uint32_t)((2 * (n_max / 4) + 2) * BM * 8 + (n_max + 1) * BM * 8);
+  return (uint32_t)((2 * (n_max / 4) + 2) * BM * 8 + (n_max + 1) * BM * 8 + (tri_blocks(n_max) + 15) / 16 * 16);
 }
 // Two blocks or more per SM.
 constexpr uint32_t kTriBasisSmem = 110 * 1024;
 
+// cos and sin of a fraction of a turn (its upper 32 bits) to float32 accuracy: the nearest quarter turn
+// taken off, Taylor polynomials of the rest.  A third of the fixed-point rotation's instructions,
+// and every multiple of the angle is evaluated by itself.
+__device__ __forceinline__ float2 turn_cos_sin(uint32_t turn) {
+  const uint32_t k = (turn + 0x20000000u) >> 30;
+  const float x = (float)(int32_t)(turn - (k << 30)) * 1.4629180792671596e-9f;  // 2 pi / 2^32
+  const float u = x * x;
+  const float s = fmaf(x * u, fmaf(u, fmaf(u, fmaf(u, 1.0f / 362880, -1.0f / 5040), 1.0f / 120), -1.0f / 6), x);
+  const float c = fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.0f / 40320, -1.0f / 720), 1.0f / 24), -0.5f), 1.0f);
+  const float a = (k & 1u) ? s : c, b = (k & 1u) ? c : s;
+  return make_float2(__uint_as_float(__float_as_uint(a) ^ (((k + 1u) & 2u) << 30)),
+                     __uint_as_float(__float_as_uint(b) ^ ((k & 2u) << 30)));
+}
+
 template <bool TF32, bool SLOW>
 __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA, uint32_t row, double rho, double th,
-                                              uint64_t* st, float2* an) {
+                                              uint64_t* st, float2* an, const uint8_t* whole) {
   using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
   constexpr int UNIT = TF32 ? 4 : 8;
   const int n_max = a.n_max, H = n_max / 2;
   TriPoint tp = {};
   if constexpr (!SLOW) {
     tp = tri_point((uint64_t)__double_as_longlong(rho));
-    int64_t ci, si;
-    tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
-    const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
-    TriTrig c = tri_split(1ll << 62), s = tri_split(0);
-    for (int m = 0; m <= n_max; ++m) {
-      // 2^-31 of the angle's word, 2^-30 of the radial one.
-      an[(size_t)m * BM] = make_float2((float)c.hi * 0x1p-61f, (float)s.hi * 0x1p-61f);
-      tri_rotate(c, s, c1, s1);
+    const uint64_t turn = tri_turn((uint64_t)__double_as_longlong(th));
+    uint64_t t = 1ull << 31;
+    for (int m = 0; m <= n_max; ++m, t += turn) {
+      const float2 g = turn_cos_sin((uint32_t)(t >> 32));
+      an[(size_t)m * BM] = make_float2(g.x * 0x1p-30f, g.y * 0x1p-30f);  // the radial word's 2^-30
     }
   } else {
     double s1, c1, c = 1.0, s = 0.0;
@@ -402,11 +413,28 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
   }
   int k_full = 0, k_tail = 8 * a.full;
   Pack16 hi, lo;
-  auto at = [&](int k) {  // byte offset of a unit's first position
+  auto at = [&](int k, uint32_t r) {  // a unit's place in row r
     uint8_t* chunk = gA + (size_t)(k / C::BK) * C::A_CHUNK;
-    if constexpr (TF32) return chunk + ptx::sw_offset_b32<C::ROW>(row, (uint32_t)(k % C::BK));
-    else return chunk + ptx::sw_offset_b16<C::ROW>(row, (uint32_t)(k % C::BK));
+    if constexpr (TF32) return chunk + ptx::sw_offset_b32<C::ROW>(r, (uint32_t)(k % C::BK));
+    else return chunk + ptx::sw_offset_b16<C::ROW>(r, (uint32_t)(k % C::BK));
   };
+  // Two neighbouring units (the halves of a 32-byte sector) of every row of the warp: lanes exchange in
+  // pairs so that each store fills whole sectors of 16 rows instead of halves of 32 (a store's cost is
+  // the lines that it touches).
+  const uint32_t odd = row & 1u;
+  auto store_pair = [&](int k, uint32_t part, const uint32_t (&x)[4], const uint32_t (&y)[4]) {
+    uint32_t e[4], o[4];  // the even row's half and the odd row's half that this lane stores
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? x[i] : y[i], 1);
+      e[i] = odd ? got : x[i];
+      o[i] = odd ? y[i] : got;
+    }
+    const int ku = k + (odd ? UNIT : 0);
+    *reinterpret_cast<uint4*>(at(ku, row & ~1u) + part) = make_uint4(e[0], e[1], e[2], e[3]);
+    *reinterpret_cast<uint4*>(at(ku, row | 1u) + part) = make_uint4(o[0], o[1], o[2], o[3]);
+  };
+  uint32_t wait_h[4], wait_l[4];  // BF16x3: the first unit of a pair
   auto tail = [&](float z) {
     if constexpr (TF32) {
       hi.push32(__float_as_uint(to_tf32(z)));
@@ -416,7 +444,7 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
       lo.push16(bf16x2_bits(z - __uint_as_float(h << 16), 0.0f) & 0xffffu);
     }
     if (++k_tail % UNIT == 0) {
-      uint8_t* dst = at(k_tail - UNIT);
+      uint8_t* dst = at(k_tail - UNIT, row);
       hi.store(dst);
       if constexpr (!TF32) lo.store(dst + C::A_PART);
     }
@@ -428,7 +456,6 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
     uint64_t l0 = SLOW ? 0ull : kTriZero, l1 = l0;
     uint64_t dg = A == 0 ? (SLOW ? (uint64_t)__double_as_longlong(-1.0) : 0ull) : l0;
     for (int B = 0; B <= nb; ++B, ++block) {
-      const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
       uint64_t* sr = st + (size_t)(2 * B) * BM;
       const uint64_t u0 = B < A ? sr[0] : l0, u1 = B < A ? sr[BM] : l1;
       uint64_t e00, e01, e10, e11;
@@ -466,12 +493,15 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
       const float2 mid = an[(size_t)m0 * BM], low = an[(size_t)max(m0 - 1, 0) * BM], top = an[(size_t)min(m0 + 1, n_max) * BM];
       const float z[8] = {f[0] * mid.x, f[1] * low.x, f[2] * top.x, f[3] * mid.x,
                           f[0] * mid.y, f[1] * low.y, f[2] * top.y, f[3] * mid.y};
-      if ((jc.x | jc.y | jc.z | jc.w | js.x | js.y | js.z | js.w) >= 0) {
+      if (whole[block]) {
         if constexpr (TF32) {
+          uint32_t x[4], y[4];
 #pragma unroll
-          for (int i = 0; i < 2; ++i)
-            *reinterpret_cast<float4*>(at(k_full + 4 * i)) =
-                make_float4(to_tf32(z[4 * i]), to_tf32(z[4 * i + 1]), to_tf32(z[4 * i + 2]), to_tf32(z[4 * i + 3]));
+          for (int i = 0; i < 4; ++i) {
+            x[i] = __float_as_uint(to_tf32(z[i]));
+            y[i] = __float_as_uint(to_tf32(z[4 + i]));
+          }
+          store_pair(k_full, 0, x, y);
         } else {
           uint32_t h[4], l[4];
 #pragma unroll
@@ -479,12 +509,24 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
             h[i] = bf16x2_bits(z[2 * i], z[2 * i + 1]);
             l[i] = bf16x2_bits(z[2 * i] - __uint_as_float(h[i] << 16), z[2 * i + 1] - __uint_as_float(h[i] & 0xffff0000u));
           }
-          uint8_t* dst = at(k_full);
-          *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-          *reinterpret_cast<uint4*>(dst + C::A_PART) = make_uint4(l[0], l[1], l[2], l[3]);
+          if (k_full & 8) {
+            store_pair(k_full - 8, 0, wait_h, h);
+            store_pair(k_full - 8, C::A_PART, wait_l, l);
+          } else if (k_full + 8 == 8 * a.full) {  // the last one, without a partner
+            uint8_t* dst = at(k_full, row);
+            *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(dst + C::A_PART) = make_uint4(l[0], l[1], l[2], l[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              wait_h[i] = h[i];
+              wait_l[i] = l[i];
+            }
+          }
         }
         k_full += 8;
       } else {
+        const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
         const int32_t j[8] = {jc.x, jc.y, jc.z, jc.w, js.x, js.y, js.z, js.w};
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -500,16 +542,24 @@ __global__ void __launch_bounds__(BM) tri_basis_kernel(TriBasisArgs a) {
   using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
   extern __shared__ uint64_t tri_basis_mem[];
   uint64_t* st = tri_basis_mem + threadIdx.x;
-  float2* an = reinterpret_cast<float2*>(tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM) + threadIdx.x;
+  float2* angles = reinterpret_cast<float2*>(tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM);
+  float2* an = angles + threadIdx.x;
+  // Which blocks have all their modes (a load per block would stall on its latency).
+  uint8_t* whole = reinterpret_cast<uint8_t*>(angles + (size_t)(a.n_max + 1) * BM);
+  for (int i = threadIdx.x; i < tri_blocks(a.n_max); i += BM) {
+    const int4 jc = __ldg(reinterpret_cast<const int4*>(a.perm) + 2 * i), js = __ldg(reinterpret_cast<const int4*>(a.perm) + 2 * i + 1);
+    whole[i] = (jc.x | jc.y | jc.z | jc.w | js.x | js.y | js.z | js.w) >= 0;
+  }
+  __syncthreads();
   const int64_t p = (a.mt_base + blockIdx.x) * BM + threadIdx.x;
   const bool valid = p < a.P;
   const double rho = valid ? a.r[p] : 0.0, th = valid ? a.theta[p] : 0.0;
   const uint32_t e = ((uint32_t)__double2hiint(th) >> 20) & 0x7ffu;
   uint8_t* gA = a.A + (size_t)blockIdx.x * a.KC * C::A_CHUNK;
   if (__any_sync(0xffffffffu, !(rho >= 0.0 && rho <= 1.0 && e < (uint32_t)kTriAngleExponent)))
-    tri_basis_row<TF32, true>(a, gA, threadIdx.x, rho, th, st, an);
+    tri_basis_row<TF32, true>(a, gA, threadIdx.x, rho, th, st, an, whole);
   else
-    tri_basis_row<TF32, false>(a, gA, threadIdx.x, rho, th, st, an);
+    tri_basis_row<TF32, false>(a, gA, threadIdx.x, rho, th, st, an, whole);
 }
 
 struct CoeffArgs {
