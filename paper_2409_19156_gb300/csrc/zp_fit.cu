@@ -222,8 +222,8 @@ __global__ void __launch_bounds__(256) chol_update_kernel(double* A, int J, int 
 // Column c of the factor divided by its pivot, below the diagonal (L = M diag(d) with M unit lower).
 __global__ void __launch_bounds__(128) unit_lower_kernel(double* L, int J) {
   const int c = blockIdx.x;
-  const double rd = 1.0 / L[(size_t)c + (size_t)c * J];
-  for (int t = c + 1 + (int)threadIdx.x; t < J; t += blockDim.x) L[(size_t)t + (size_t)c * J] *= rd;
+  const double d = L[(size_t)c + (size_t)c * J];
+  for (int t = c + 1 + (int)threadIdx.x; t < J; t += blockDim.x) L[(size_t)t + (size_t)c * J] /= d;
 }
 
 // Solves M diag(d^2) M^T X = B for kSolveCols columns of B per CTA (B column-major J x S) and stores X
@@ -314,8 +314,8 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const double* __restric
     __syncthreads();
     if (i == blocks - 1) {  // between the passes: divide by the squared pivots
       for (int t = tid; t < J; t += blockDim.x) {
-        const double d = M[(size_t)t + (size_t)t * J], r = 1.0 / (d * d);
-        for (int k = 0; k < kSolveCols; ++k) y[(size_t)k * JP + t] *= r;
+        const double d = M[(size_t)t + (size_t)t * J];
+        for (int k = 0; k < kSolveCols; ++k) y[(size_t)k * JP + t] = y[(size_t)k * JP + t] / d / d;
       }
       __syncthreads();
     }

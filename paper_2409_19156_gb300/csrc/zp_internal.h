@@ -137,10 +137,13 @@ zp_status check_plan_device(const zp_plan* plan);
 // phase_ms: NULL, or [2] receiving the device time of the point preparation and of the walk
 // (events around each launch; the stream is synchronised).  rowmax: NULL, or (a walk of Z:
 // theta given, max_deriv 0) [modes] words, zeroed by the caller, receiving each output row's
-// largest |value| high word << 32.
+// largest |value| high word << 32.  unweighted (with rowmax): the rows hold Z over their modes' recursion
+// weights, for sums over the points that launch_weight_rows completes.
 zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta, int64_t n_points,
                       int max_deriv, double* out, double* out_dtheta, cudaStream_t stream,
-                      float* phase_ms = nullptr, unsigned long long* rowmax = nullptr);
+                      float* phase_ms = nullptr, unsigned long long* rowmax = nullptr, bool unweighted = false);
+// Multiplies row j of C [n_modes][S] by mode j's weight, which an unweighted walk leaves out.
+zp_status launch_weight_rows(const zp_plan* plan, int64_t S, double* C, cudaStream_t stream);
 zp_status launch_per_mode(const zp_plan* plan, const double* r, int64_t n_points, double* out,
                           cudaStream_t stream);
 

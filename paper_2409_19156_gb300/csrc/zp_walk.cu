@@ -326,6 +326,94 @@ __global__ void __launch_bounds__(TPB) walk_kernel(WalkArgs a) {
   }
 }
 
+// Z without its weights, Q_N cos/sin(m theta) = Z / W0_N, for contractions over the points (whose
+// results take the weight): the recursion is linear in its seeds, so walked from the seeds times cos and
+// times sin it gives both products with one FMA each, three float64 operations per (n, |m|) and point
+// instead of five (g_N shared by the two).  Stores and row maxima as walk_kernel's at k = 0.
+template <bool VEC, int TPB>
+__global__ void __launch_bounds__(TPB) walk_unweighted_kernel(WalkArgs a) {
+  constexpr int PPT = TPB == kThreads ? kPPT : 1;
+  extern __shared__ double smem[];
+  const Column col = a.cols[blockIdx.y];
+  const int n_rows = kHeaderRows + col.n_steps;
+  double2* ab = reinterpret_cast<double2*>(smem);  // (A_N, B_N) after the header
+  int32_t* sptr = reinterpret_cast<int32_t*>(smem + (size_t)2 * n_rows);
+  const double* h = a.table + (size_t)col.table_row * kRow;
+  for (int i = threadIdx.x; i < n_rows; i += TPB) ab[i] = *reinterpret_cast<const double2*>(h + (size_t)i * kRow);
+  for (int i = threadIdx.x; i <= col.n_steps; i += TPB) sptr[i] = a.slot_ptr[col.slot_base + i];
+  __syncthreads();
+  const int64_t p0 = ((int64_t)blockIdx.x * TPB + (int64_t)threadIdx.x) * PPT;
+  if (p0 >= a.P) return;
+  const bool two = PPT == 2 && p0 + 1 < a.P;
+  const int m = col.m;
+  double u[PPT], Tc[PPT], Ts[PPT], Sc[PPT], Ss[PPT];
+#pragma unroll
+  for (int i = 0; i < PPT; ++i) {
+    const int64_t p = (i == 0 || two) ? p0 + i : p0;
+    const double rho = a.r[p];
+    u[i] = rho * rho;
+    double c = 1.0, s = 0.0, pm, pm2;
+    if (a.cs != nullptr) {
+      c = a.cs[(int64_t)m * a.P + p];
+      s = a.sn[(int64_t)m * a.P + p];
+    } else if (m != 0) {
+      sincos((double)m * a.theta[p], &s, &c);
+    }
+    if (a.pw != nullptr) {
+      pm = a.pw[(int64_t)m * a.P + p];
+      pm2 = a.pw[(int64_t)(m + 2) * a.P + p];
+    } else {
+      pm = pow_uint(rho, m);
+      pm2 = pm * u[i];
+    }
+    // Q_0 = rho^m, Q_1 = (m + 2) rho^(m+2) - (m + 1) rho^m.
+    const double q1 = fma(__ldg(h + 4), pm2, -(__ldg(h + 8) * pm));
+    Tc[i] = pm * c;
+    Ts[i] = pm * s;
+    Sc[i] = q1 * c;
+    Ss[i] = q1 * s;
+  }
+  auto store_step = [&](int N, const double (&c)[PPT], const double (&s)[PPT]) {
+    for (int i = sptr[N]; i < sptr[N + 1]; ++i) {
+      const uint32_t code = (uint32_t)__ldg(a.slot_idx + i);
+      const int64_t j = (int64_t)(code & 0x7fffffffu);
+      const bool is_sin = (code >> 31) != 0;
+      const double v0 = is_sin ? s[0] : c[0], v1 = is_sin ? s[PPT - 1] : c[PPT - 1];
+      store_pts<PPT>(a.out + j * a.P, p0, v0, v1, two, VEC);
+      uint32_t hw = (uint32_t)__double2hiint(v0) & 0x7fffffffu;
+      if (PPT == 2 && two) hw = max(hw, (uint32_t)__double2hiint(v1) & 0x7fffffffu);
+      const unsigned mask = __activemask();
+      const uint32_t mx = __reduce_max_sync(mask, hw);
+      if ((int)(threadIdx.x & 31u) == __ffs((int)mask) - 1) atomicMax(a.rowmax + j, (unsigned long long)mx << 32);
+    }
+  };
+  store_step(0, Tc, Ts);
+  if (col.n_steps < 2) return;
+  store_step(1, Sc, Ss);
+  for (int N = 2; N < col.n_steps; ++N) {
+    const double2 AB = ab[kHeaderRows + N];
+#pragma unroll
+    for (int i = 0; i < PPT; ++i) {
+      const double g = fma(AB.x, u[i], -AB.y);
+      const double nc = fma(g, Sc[i], -Tc[i]), ns = fma(g, Ss[i], -Ts[i]);
+      Tc[i] = Sc[i];
+      Ts[i] = Ss[i];
+      Sc[i] = nc;
+      Ss[i] = ns;
+    }
+    store_step(N, Sc, Ss);
+  }
+}
+
+// The weights that walk_unweighted_kernel leaves out, applied to rows of C [J][S].
+__global__ void __launch_bounds__(256) weight_rows_kernel(const Column* cols, const double* table, const int32_t* mode_col,
+                                                          const int32_t* mode_N, int64_t J, int64_t S, double* C) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < J * S; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t j = i / S;
+    C[i] *= table[((size_t)cols[mode_col[j]].table_row + kHeaderRows + mode_N[j]) * kRow + 3];
+  }
+}
+
 // Algorithm 2 of Sec. 3: one thread per (point, mode), each running its own recursion to
 // its own degree and storing only the last value (k = 0).  Comparison kernel.
 __global__ void __launch_bounds__(kThreads) per_mode_kernel(const Column* cols, const double* table,
@@ -410,10 +498,11 @@ struct WalkTimer {
 
 zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta, int64_t n_points, int max_deriv,
                       double* out, double* out_dtheta, cudaStream_t stream, float* phase_ms,
-                      unsigned long long* rowmax) {
+                      unsigned long long* rowmax, bool unweighted) {
   if (phase_ms) phase_ms[0] = phase_ms[1] = 0.0f;
   if (rowmax && (max_deriv != 0 || theta == nullptr))
     return set_error(ZP_ERR_INVALID_ARG, "row maxima are formed for walks of Z at k = 0 only");
+  if (unweighted && !rowmax) return set_error(ZP_ERR_INVALID_ARG, "the unweighted walk forms row maxima");
   if (n_points == 0 || plan->n_modes == 0) return ZP_OK;
   WalkTimer timer(phase_ms, stream);
   WalkArgs a;
@@ -436,7 +525,7 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
   const int64_t n_cols = (int64_t)plan->cols.size();
   // Mode lists that fill their triangle take the walk over neighbouring m for the points that make
   // whole waves of it.
-  a.p_first = tri_walk_points(plan, n_points, max_deriv, theta != nullptr, out_dtheta != nullptr, sms);
+  a.p_first = unweighted ? 0 : tri_walk_points(plan, n_points, max_deriv, theta != nullptr, out_dtheta != nullptr, sms);
   if (a.p_first > 0) {
     ZP_TRY(launch_tri_walk(plan, r, theta, n_points, a.p_first, max_deriv, out, out_dtheta, rowmax, stream));
     if (a.p_first == n_points) {
@@ -485,6 +574,17 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
     a.cs = cs;
     a.sn = sn;
   }
+  if (unweighted) {
+    const size_t bytes = (size_t)2 * (kHeaderRows + plan->max_steps) * sizeof(double) +
+                         (size_t)(plan->max_steps + 1) * sizeof(int32_t);
+    if (small && vec) walk_unweighted_kernel<true, kThreadsSmall><<<grid, kThreadsSmall, bytes, stream>>>(a);
+    else if (small) walk_unweighted_kernel<false, kThreadsSmall><<<grid, kThreadsSmall, bytes, stream>>>(a);
+    else if (vec) walk_unweighted_kernel<true, kThreads><<<grid, kThreads, bytes, stream>>>(a);
+    else walk_unweighted_kernel<false, kThreads><<<grid, kThreads, bytes, stream>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "walk_unweighted_kernel launch");
+    timer.mark(2);
+    return timer.finish();
+  }
   // Duplicated modes: some (column, N) step stores to more than two outputs.
   bool dup = false;
   for (size_t i = 0; i + 1 < plan->slot_ptr.size() && !dup; ++i) dup = plan->slot_ptr[i + 1] - plan->slot_ptr[i] > 2;
@@ -498,6 +598,15 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
   if (e != cudaSuccess) return cuda_error(e, "walk_kernel launch");
   timer.mark(2);
   return timer.finish();
+}
+
+zp_status launch_weight_rows(const zp_plan* plan, int64_t S, double* C, cudaStream_t stream) {
+  const int64_t blocks = std::min<int64_t>((plan->n_modes * S + 255) / 256, 1 << 16);
+  if (blocks == 0) return ZP_OK;
+  weight_rows_kernel<<<(unsigned)blocks, 256, 0, stream>>>(plan->dev.cols, plan->dev.table, plan->dev.mode_col,
+                                                          plan->dev.mode_N, plan->n_modes, S, C);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? ZP_OK : cuda_error(e, "weight_rows_kernel launch");
 }
 
 zp_status launch_per_mode(const zp_plan* plan, const double* r, int64_t n_points, double* out, cudaStream_t stream) {
