@@ -1,0 +1,52 @@
+// cos and sin of the multiples of an angle in float64, on the integer pipe where that serves.
+#pragma once
+
+#include "zp_tri.h"
+
+namespace zp {
+
+// v 2^-62 as a float64, rounded to nearest, by integer operations.
+__device__ __forceinline__ double from_fixed62(int64_t v) {
+  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a);
+  const uint64_t m = a << lz;  // top bit set
+  uint64_t b = ((m >> 11) & 0xfffffffffffffull) | ((uint64_t)(1023 - 62 + 63 - lz) << 52);
+  b += (m >> 10) & 1;
+  return __longlong_as_double((long long)(b | ((uint64_t)v & (1ull << 63))));
+}
+
+// Calls f(m, cos m theta, sin m theta) for m = 0 .. m_max.  In fixed point (absolute errors below 2^-57;
+// a float64 product m theta alone rounds by up to 2^-53 m theta) unless the angle is so small that
+// sin(m theta) needs relative accuracy, or out of range: then by angle addition in float64, restarted
+// from sincos at every 16th m.
+template <typename F>
+__device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
+  const double mag = fabs(th);
+  if (mag >= 1.0 / 128 && mag < 2048.0) {
+    int64_t ci, si;
+    tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
+    const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
+    TriTrig c = tri_split(1ll << 62), s = tri_split(0);
+    f(0, 1.0, 0.0);
+    for (int m = 1; m <= m_max; ++m) {
+      tri_rotate(c, s, c1, s1);
+      f(m, from_fixed62((int64_t)c.hi * (1ll << 31) + c.lo), from_fixed62((int64_t)s.hi * (1ll << 31) + s.lo));
+    }
+  } else {
+    double s1, c1, c = 1.0, s = 0.0;
+    sincos(th, &s1, &c1);
+    for (int m = 0; m <= m_max; ++m) {
+      if (m % 16 == 0) {
+        if (m > 0) sincos((double)m * th, &s, &c);
+      } else {
+        const double cn = fma(c, c1, -s * s1);
+        s = fma(s, c1, c * s1);
+        c = cn;
+      }
+      f(m, c, s);
+    }
+  }
+}
+
+}  // namespace zp

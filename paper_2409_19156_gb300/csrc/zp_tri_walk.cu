@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "zp_angles.cuh"
 #include "zp_api_common.h"
 #include "zp_internal.h"
 #include "zp_series_internal.h"
@@ -47,49 +48,6 @@ __host__ __device__ constexpr uint32_t walk_smem(int n_max, int kmax, bool ang) 
   return (uint32_t)(rows_of(n_max) * (kmax + 1) * W * 8 + (n_max + 3) * 8 + (ang ? (n_max + 1) * W * 16 : 0));
 }
 
-// v 2^-62 as a float64, rounded to nearest, by integer operations.
-__device__ __forceinline__ double from_fixed62(int64_t v) {
-  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
-  if (a == 0) return 0.0;
-  const int lz = __clzll((long long)a);
-  const uint64_t m = a << lz;  // top bit set
-  uint64_t b = ((m >> 11) & 0xfffffffffffffull) | ((uint64_t)(1023 - 62 + 63 - lz) << 52);
-  b += (m >> 10) & 1;
-  return __longlong_as_double((long long)(b | ((uint64_t)v & (1ull << 63))));
-}
-
-// cos and sin(m theta), m = 0 .. n_max, of this thread's point.  In fixed point (absolute errors below
-// 2^-57) unless the angle is so small that sin(m theta) needs relative accuracy, or out of its range:
-// then by angle addition in float64, restarted from sincos at every 16th m.
-__device__ __forceinline__ void angle_rows(double th, int n_max, double2* an) {
-  const double mag = fabs(th);
-  if (mag >= 1.0 / 128 && mag < 2048.0) {
-    int64_t ci, si;
-    tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
-    const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
-    TriTrig c = tri_split(1ll << 62), s = tri_split(0);
-    an[0] = make_double2(1.0, 0.0);
-    for (int m = 1; m <= n_max; ++m) {
-      tri_rotate(c, s, c1, s1);
-      an[(size_t)m * W] = make_double2(from_fixed62((int64_t)c.hi * (1ll << 31) + c.lo),
-                                       from_fixed62((int64_t)s.hi * (1ll << 31) + s.lo));
-    }
-  } else {
-    double s1, c1, c = 1.0, s = 0.0;
-    sincos(th, &s1, &c1);
-    for (int m = 0; m <= n_max; ++m) {
-      if (m % 16 == 0) {
-        if (m > 0) sincos((double)m * th, &s, &c);
-      } else {
-        const double cn = fma(c, c1, -s * s1);
-        s = fma(s, c1, c * s1);
-        c = cn;
-      }
-      an[(size_t)m * W] = make_double2(c, s);
-    }
-  }
-}
-
 // KMAX: highest rho-derivative; ANG: Z instead of R; DT (with ANG): also dZ/dtheta.
 template <int KMAX, bool ANG, bool DT>
 __global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
@@ -104,7 +62,8 @@ __global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
   const int64_t p = (int64_t)blockIdx.x * W + lane;
   const bool valid = p < a.p_end;
   const double rho = valid ? a.r[p] : 0.0;
-  if constexpr (ANG) angle_rows(valid ? a.theta[p] : 0.0, n_max, an);
+  if constexpr (ANG)
+    for_each_angle(valid ? a.theta[p] : 0.0, n_max, [&](int m, double c, double s) { an[(size_t)m * W] = make_double2(c, s); });
   double* const out = a.out + p;
   double* const out_dt = DT ? a.out_dtheta + p : nullptr;
   const int64_t order = a.J * a.P;
