@@ -53,7 +53,8 @@ constexpr uint32_t kTriWalkSmem = 56 * 1024;
 int64_t tri_walk_points(const zp_plan* plan, int64_t n_points, int max_deriv, bool ang, bool dtheta, int sms);
 // Points 0 .. p_end - 1 of n_points; arguments as launch_walk.
 zp_status launch_tri_walk(const zp_plan* plan, const double* r, const double* theta, int64_t n_points, int64_t p_end,
-                          int max_deriv, double* out, double* out_dtheta, unsigned long long* rowmax, cudaStream_t stream);
+                          int max_deriv, double* out, double* out_dtheta, unsigned long long* rowmax, int sms,
+                          cudaStream_t stream);
 
 zp_status series_eval_fp64(const zp_plan* plan, const double* r, const double* theta, int64_t P,
                            const double* coeffs, int64_t S, double* out, cudaStream_t stream);

@@ -11,10 +11,17 @@
 // One warp per 32 points, one point per thread, walking 2 x 2 blocks of (a, b) = ((n+m)/2, (n-m)/2)
 // row by row; the row above (every lane of its derivatives) is kept in shared memory, private to the
 // thread, so nothing synchronises.  Bound: float64 issue (a warp's operation holds its scheduler's
-// pipe for 64 cycles), so a warp per scheduler is enough, and the shared memory may be large; the
-// stores are whole 128-byte lines per warp.  Measured against the column form: radial set n <= 100,
-// k <= 3, 1e5 points 6.32 -> 4.62 ms; Z and dZ/drho with dZ/dtheta, n <= 32, 99991 points 836 -> 631 us.  cos / sin(m theta) come from the fixed-point angle
-// functions on the integer pipe, which is idle here.
+// pipe for 64 cycles); the stores are whole 128-byte lines per warp.  cos / sin(m theta) come from
+// the fixed-point angle functions on the integer pipe, which is idle here.
+//
+// With the whole row in shared memory, high degrees leave room for one warp per scheduler, which
+// keeps the pipe two thirds busy: the instructions between two float64 operations are not hidden.
+// The wide form (radial, k >= 2) holds the row's two highest derivative lanes in tensor memory (each
+// warp reads its own 32 lanes of it), so that two warps per scheduler fit: eight in a block, one
+// block per SM.  The next block's lanes are read under the operations of this one.
+//
+// Measured against the column form: radial set n <= 100, k <= 3, 1e5 points 6.32 -> 3.66 ms (4.62
+// with one warp per scheduler); Z and dZ/drho with dZ/dtheta, n <= 32, 99991 points 836 -> 631 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,19 +30,24 @@
 #include "zp_angles.cuh"
 #include "zp_api_common.h"
 #include "zp_internal.h"
+#include "zp_ptx.cuh"
 #include "zp_series_internal.h"
 #include "zp_tri.h"
 
 namespace zp {
 namespace {
 
-constexpr int W = 32;  // points per block (one warp)
+constexpr int W = 32;           // points per warp
+constexpr int kWideWarps = 8;   // warps of a block that keeps part of its rows in tensor memory
+constexpr int kWideLanes = 2;   // its value lanes there (the highest derivatives)
+constexpr uint32_t kMaxBlockSmem = 232448 - 64, kSmemPerSm = 233472, kSmemPerBlock = 1024;
+constexpr int kWideCols = 256;  // tensor memory columns per warp: two warps share a quadrant's 512
 
 struct TriWalkArgs {
   const int32_t* perm;  // modes of every position (zp_tri.h), -1 for none
   const double* r;
   const double* theta;
-  int64_t p_end;  // points 0 .. p_end - 1 of P
+  int64_t p_begin, p_end;  // points p_begin .. p_end - 1 of P
   int64_t P, J;
   double* out;
   double* out_dtheta;
@@ -48,18 +60,49 @@ __host__ __device__ constexpr uint32_t walk_smem(int n_max, int kmax, bool ang) 
   return (uint32_t)(rows_of(n_max) * (kmax + 1) * W * 8 + (n_max + 3) * 8 + (ang ? (n_max + 1) * W * 16 : 0));
 }
 
-// KMAX: highest rho-derivative; ANG: Z instead of R; DT (with ANG): also dZ/dtheta.
-template <int KMAX, bool ANG, bool DT>
-__global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
+constexpr uint32_t wide_smem(int n_max, int kmax) {
+  return (uint32_t)(rows_of(n_max) * (kmax + 1 - kWideLanes) * kWideWarps * W * 8 + (n_max + 3) * 8);
+}
+// Whether the wide form fits (tensor memory columns and shared memory of one block per SM) and the
+// one-warp form leaves fewer than six warps per SM (1e5 points, wide against one-warp form: k <= 3, four
+// per SM, n <= 100: 3.71 against 4.62 ms; five per SM, n <= 72, k <= 3: 2.02 against 2.14 ms, and n <= 100,
+// k <= 2: 2.80 against 2.91 ms).
+constexpr bool wide_fits(int n_max, int kmax, bool ang) {
+  return !ang && kmax >= 2 && rows_of(n_max) * kWideLanes * 2 <= kWideCols && wide_smem(n_max, kmax) <= kMaxBlockSmem &&
+         walk_smem(n_max, kmax, false) + kSmemPerBlock > kSmemPerSm / 6;
+}
+
+// KMAX: highest rho-derivative; ANG: Z instead of R; DT (with ANG): also dZ/dtheta; WIDE: eight warps
+// per block, the row's two highest derivative lanes in tensor memory.
+template <int KMAX, bool ANG, bool DT, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kWideWarps * W : W) tri_walk_kernel(TriWalkArgs a) {
+  static_assert(!WIDE || (!ANG && KMAX >= 2));
   extern __shared__ double tri_smem[];
-  constexpr int L = KMAX + 1;
-  const int lane = threadIdx.x, n_max = a.n_max, H = n_max / 2;
+  __shared__ uint32_t tmem_base;
+  constexpr int L = KMAX + 1, LS = WIDE ? L - kWideLanes : L;  // lanes; those in shared memory
+  constexpr int kWarps = WIDE ? kWideWarps : 1;
+  // Four blocks per iteration: no register moves between them (radial set n <= 100, k <= 3, 1e5 points
+  // 4.12 -> 3.66 ms); Z was slower with it (0.63 -> 0.65 ms).
+  constexpr int kUnroll = ANG ? 1 : 4;
+  const int lane = threadIdx.x % W, warp = threadIdx.x / W, n_max = a.n_max, H = n_max / 2;
   double2* an = reinterpret_cast<double2*>(tri_smem) + lane;  // [m][lane]
-  double* st = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + lane;  // [b][k][lane]
-  double* num = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)rows_of(n_max) * L * W;  // 0, 1, 2, ..
-  for (int i = lane; i < n_max + 3; i += W) num[i] = (double)i;
-  __syncwarp();
-  const int64_t p = (int64_t)blockIdx.x * W + lane;
+  double* st = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)warp * rows_of(n_max) * LS * W + lane;  // [b][k][lane]
+  double* num = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)kWarps * rows_of(n_max) * LS * W;  // 0, 1, 2, ..
+  for (int i = threadIdx.x; i < n_max + 3; i += kWarps * W) num[i] = (double)i;
+  uint32_t tm = 0;  // [b / 2][row of two][k][low, high word] of this thread's lane
+  if constexpr (WIDE) {
+    if (warp == 0) {
+      ptx::tmem_alloc(&tmem_base, 2 * kWideCols);
+      ptx::tmem_relinquish();
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    tm = tmem_base + ((uint32_t)(warp % 4) << 21) + (uint32_t)(warp / 4) * kWideCols;
+  } else {
+    __syncwarp();
+  }
+  const int64_t p = a.p_begin + ((int64_t)blockIdx.x * kWarps + warp) * W + lane;
   const bool valid = p < a.p_end;
   const double rho = valid ? a.r[p] : 0.0;
   if constexpr (ANG)
@@ -111,14 +154,37 @@ __global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
 #pragma unroll
     for (int k = 0; k < L; ++k) l0[k] = l1[k] = dg[k] = 0.0;
     if (A == 0) dg[0] = -1.0;
+    uint32_t v[8] = {};  // the row above in tensor memory
+    if constexpr (WIDE) {
+      if (A > 0) ptx::tmem_ld_32x32b_x8(tm, v);
+    }
+#pragma unroll kUnroll
     for (int B = 0; B <= nb; ++B, ++block) {
+      if constexpr (WIDE) __syncwarp();
       const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
-      double* row = st + (size_t)(2 * B) * L * W;
+      double* row = st + (size_t)(2 * B) * LS * W;
       double u0[L], u1[L], e00[L], e01[L], e10[L], e11[L];
 #pragma unroll
-      for (int k = 0; k < L; ++k) {
+      for (int k = 0; k < LS; ++k) {
         u0[k] = B < A ? row[k * W] : l0[k];
-        u1[k] = B < A ? row[(L + k) * W] : l1[k];
+        u1[k] = B < A ? row[(LS + k) * W] : l1[k];
+      }
+      if constexpr (WIDE) {
+        if (B < A) {
+          ptx::tmem_ld_wait(v);
+#pragma unroll
+          for (int k = 0; k < kWideLanes; ++k) {
+            u0[LS + k] = __hiloint2double((int)v[2 * k + 1], (int)v[2 * k]);
+            u1[LS + k] = __hiloint2double((int)v[2 * k + 5], (int)v[2 * k + 4]);
+          }
+        } else {
+#pragma unroll
+          for (int k = LS; k < L; ++k) {
+            u0[k] = l0[k];
+            u1[k] = l1[k];
+          }
+        }
+        if (B + 1 < A && B < nb) ptx::tmem_ld_32x32b_x8(tm + 8 * B + 8, v);  // the next block's, under this one's operations
       }
       const int n0 = 2 * (A + B), m0 = 2 * (A - B);
       const double nd0 = num[n0], nd1 = num[n0 + 1], nd2 = num[n0 + 2];
@@ -138,39 +204,67 @@ __global__ void __launch_bounds__(W) tri_walk_kernel(TriWalkArgs a) {
       element(e11, e01, e10, e00, nd2);
 #pragma unroll
       for (int k = 0; k < L; ++k) {
-        row[k * W] = e10[k];
-        row[(L + k) * W] = e11[k];
+        if (k < LS) {
+          row[k * W] = e10[k];
+          row[(LS + k) * W] = e11[k];
+        }
         dg[k] = u1[k];
         l0[k] = e01[k];
         l1[k] = e11[k];
+      }
+      if constexpr (WIDE) {
+        auto lo = [](double x) { return (uint32_t)__double2loint(x); };
+        auto hi = [](double x) { return (uint32_t)__double2hiint(x); };
+        ptx::tmem_st_32x32b_x4<0>(tm + 8 * B, lo(e10[LS]), hi(e10[LS]), lo(e10[LS + 1]), hi(e10[LS + 1]));
+        ptx::tmem_st_32x32b_x4<4>(tm + 8 * B, lo(e11[LS]), hi(e11[LS]), lo(e11[LS + 1]), hi(e11[LS + 1]));
       }
       emit(e00, jc.x, js.x, m0);
       emit(e01, jc.y, js.y, max(m0 - 1, 0));
       emit(e10, jc.z, js.z, min(m0 + 1, n_max));
       emit(e11, jc.w, js.w, m0);
     }
+    if constexpr (WIDE) {  // before the next row's reads
+      __syncwarp();
+      ptx::tmem_st_wait();
+    }
+  }
+  if constexpr (WIDE) {
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == 0) ptx::tmem_dealloc(tmem_base, 2 * kWideCols);
   }
 }
 
-template <int KMAX, bool ANG, bool DT>
-cudaError_t launch(const TriWalkArgs& a, unsigned blocks, uint32_t smem, cudaStream_t st) {
+template <int KMAX, bool ANG, bool DT, bool WIDE>
+cudaError_t launch(const TriWalkArgs& a, uint32_t smem, cudaStream_t st) {
   static DeviceMemo<int> memo;
   int set = 0;
   const zp_status s = memo.get(&set, [](int* x) -> zp_status {
     *x = 1;
-    const cudaError_t e = cudaFuncSetAttribute(tri_walk_kernel<KMAX, ANG, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kTriWalkSmem);
+    const cudaError_t e = cudaFuncSetAttribute(tri_walk_kernel<KMAX, ANG, DT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(WIDE ? kMaxBlockSmem : kTriWalkSmem));
     return e == cudaSuccess ? ZP_OK : cuda_error(e, "triangle walk set-up");
   });
   if (s != ZP_OK) return cudaErrorInvalidValue;
-  tri_walk_kernel<KMAX, ANG, DT><<<blocks, W, smem, st>>>(a);
+  constexpr int kPoints = WIDE ? kWideWarps * W : W;
+  tri_walk_kernel<KMAX, ANG, DT, WIDE><<<(unsigned)((a.p_end - a.p_begin + kPoints - 1) / kPoints), kPoints, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 template <int KMAX>
-cudaError_t launch_k(const TriWalkArgs& a, unsigned blocks, uint32_t smem, cudaStream_t st) {
-  if (a.theta == nullptr) return launch<KMAX, false, false>(a, blocks, smem, st);
-  return a.out_dtheta ? launch<KMAX, true, true>(a, blocks, smem, st) : launch<KMAX, true, false>(a, blocks, smem, st);
+cudaError_t launch_k(TriWalkArgs a, int64_t wide, cudaStream_t st) {
+  if constexpr (KMAX >= 2) {
+    if (wide > 0) {
+      TriWalkArgs b = a;
+      b.p_end = wide;
+      const cudaError_t e = launch<KMAX, false, false, true>(b, wide_smem(a.n_max, KMAX), st);
+      if (e != cudaSuccess || wide == a.p_end) return e;
+      a.p_begin = wide;
+    }
+  }
+  const uint32_t smem = walk_smem(a.n_max, KMAX, a.theta != nullptr);
+  if (a.theta == nullptr) return launch<KMAX, false, false, false>(a, smem, st);
+  return a.out_dtheta ? launch<KMAX, true, true, false>(a, smem, st) : launch<KMAX, true, false, false>(a, smem, st);
 }
 
 }  // namespace
@@ -187,7 +281,8 @@ int64_t tri_walk_points(const zp_plan* plan, int64_t n_points, int max_deriv, bo
   // The walk runs a warp per scheduler in whole waves of 4 sms warps; what is left over takes the
   // column form, which spreads a point over its columns.  An operation costs the walk about 4/3 of
   // the column form's time (its float64 pipe waits for shared memory and stores where the column
-  // form's eight steps overlap: radial set n <= 100, k <= 3: 440 against 622 G operations/s).
+  // form's eight steps overlap: radial set n <= 100, k <= 3, one warp per scheduler: 440 against 622 G
+  // operations/s).
   const int64_t wave = 4 * (int64_t)sms * W;
   int64_t points = n_points / wave * wave;
   const int64_t rest = n_points - points;
@@ -196,11 +291,13 @@ int64_t tri_walk_points(const zp_plan* plan, int64_t n_points, int max_deriv, bo
 }
 
 zp_status launch_tri_walk(const zp_plan* plan, const double* r, const double* theta, int64_t n_points, int64_t p_end,
-                          int max_deriv, double* out, double* out_dtheta, unsigned long long* rowmax, cudaStream_t stream) {
+                          int max_deriv, double* out, double* out_dtheta, unsigned long long* rowmax, int sms,
+                          cudaStream_t stream) {
   TriWalkArgs a;
   a.perm = plan->dev.tri_perm;
   a.r = r;
   a.theta = theta;
+  a.p_begin = 0;
   a.p_end = p_end;
   a.P = n_points;
   a.J = plan->n_modes;
@@ -210,13 +307,15 @@ zp_status launch_tri_walk(const zp_plan* plan, const double* r, const double* th
   a.n_max = plan->n_max;
   const int64_t blocks = (p_end + W - 1) / W;
   if (blocks > 0x7fffffffLL) return set_error(ZP_ERR_INVALID_ARG, "n_points too large for one launch");
-  const uint32_t smem = walk_smem(plan->n_max, max_deriv, theta != nullptr);
+  // Whole waves of eight warps per SM in the wide form, what is left over one warp per scheduler.
+  const int64_t wave = (int64_t)sms * kWideWarps * W;
+  const int64_t wide = wide_fits(plan->n_max, max_deriv, theta != nullptr) ? p_end / wave * wave : 0;
   cudaError_t e;
   switch (max_deriv) {
-    case 0: e = launch_k<0>(a, (unsigned)blocks, smem, stream); break;
-    case 1: e = launch_k<1>(a, (unsigned)blocks, smem, stream); break;
-    case 2: e = launch_k<2>(a, (unsigned)blocks, smem, stream); break;
-    default: e = launch_k<3>(a, (unsigned)blocks, smem, stream); break;
+    case 0: e = launch_k<0>(a, wide, stream); break;
+    case 1: e = launch_k<1>(a, wide, stream); break;
+    case 2: e = launch_k<2>(a, wide, stream); break;
+    default: e = launch_k<3>(a, wide, stream); break;
   }
   return e == cudaSuccess ? ZP_OK : cuda_error(e, "tri_walk_kernel launch");
 }

@@ -517,7 +517,8 @@ zp_status launch_walk(const zp_plan* plan, const double* r, const double* theta,
   // whole waves of it.
   a.p_first = unweighted ? 0 : tri_walk_points(plan, n_points, max_deriv, theta != nullptr, out_dtheta != nullptr, sms);
   if (a.p_first > 0) {
-    ZP_TRY(launch_tri_walk(plan, r, theta, n_points, a.p_first, max_deriv, out, out_dtheta, rowmax, stream));
+    ZP_TRY(launch_tri_walk(plan, r, theta, n_points, a.p_first, max_deriv, out, out_dtheta, rowmax, sms,
+                           stream));
     if (a.p_first == n_points) {
       timer.mark(2);
       return timer.finish();

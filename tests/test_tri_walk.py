@@ -122,6 +122,28 @@ def test_float64_walk_against_oracle(n_max, k, which):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_max,k", [(68, 3), (90, 2), (103, 3), (107, 3), (108, 3), (127, 2), (128, 2)])
+def test_wide_float64_walk_against_oracle(n_max, k):
+    """The form that keeps two derivative lanes in tensor memory, up to the degrees where its columns or
+    its shared memory end and the next form takes over, with a rest for the one-warp and column forms."""
+    pytest.importorskip("torch")
+    import torch
+
+    import paper_2409_19156_gb300 as zp
+    from oracle import radial as oradial
+
+    P = 60_001
+    ns, ms = inputs.radial_modes(n_max)
+    r, _ = inputs.uniform_points(P, n_max)
+    rows = np.array([0, 31, 128, 255, 256, 38_911, 38_912, 58_367, 58_368, 60_000])
+    r[[0, 31]] = [0.0, 1.0]
+    got = zp.radial(ns, ms, torch.as_tensor(r, device="cuda"), k)[:, :, rows].cpu().numpy()
+    want = np.array(oradial.radial_table(ns, ms, r[rows], k))
+    tol = 1e-11 * np.maximum(ns, 1).astype(float)[None, :, None] ** (2 * np.arange(k + 1))[:, None, None]
+    assert (np.abs(got - want) <= tol).all()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("prec,bound", [("bf16x3", 1e-4), ("tf32", 2e-3)])
 @pytest.mark.parametrize("n_max,P,S,which", [(0, 1, 1, "full"), (1, 130, 3, "full"), (7, 127, 5, "most"), (32, 700, 20, "full"),
                                              (45, 300, 257, "most"), (64, 129, 4, "full"), (70, 129, 4, "full")])
