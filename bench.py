@@ -36,18 +36,15 @@ WORKLOAD = "radial_n100"
 # the library's float64 probe (zp_probe_fp64: one wave of independent FMA chains, CUDA events).
 SMS, DP_LANES_PER_SM, SM_MAX_MHZ = 152, 2, 2070.0
 DP_OPS_PEAK_NOMINAL = SMS * DP_LANES_PER_SM * SM_MAX_MHZ * 1e6
-# Algorithmic work per (point, mode) of the k <= 3 radial workload: 14 FMA = 28 flop (the
-# unscaled recursion and its three derivative lanes).  The kernel's rescaled form issues 15
-# float64 operations per (point, mode): 1 (g) + 1 (g') + 1 + 2 + 3 + 3 (Taylor lanes 0..3) + 4
-# (stores scaled by k! w_N), every one as an FMA.
-FLOP_PER_VALUE_TUPLE = 28
-DP_OPS_PER_VALUE_TUPLE = 15
-# DRAM bytes (read + write) of one walk_kernel<3,false,true> launch at 20000 points, from one
-# ncu capture of that kernel (dram__bytes_write.sum 1.603925 GB + dram__bytes_read.sum
-# 16.961 MB: the output and one read of the power table), scaled to 100000 points (both
-# proportional to the point count).  The walk kernel has not changed since that capture (the
-# build with the step loop unrolled by eight).
-WALK_TRAFFIC_20000 = 1.603924736e9 + 16.96128e6
+# Algorithmic work per (point, mode) of the k <= 3 radial workload, by the recursion over
+# neighbouring m that its kernel runs: T_k = (R_{n-1}^{|m-1|})^(k) + (R_{n-1}^{m+1})^(k), k = 0, 1, 2
+# (3 additions), R_n^m = rho T_0 - R_{n-2}^m and (R_n^m)^(k) = n T_{k-1} + (R_{n-2}^m)^(k), k = 1, 2, 3
+# (4 FMA): 7 float64 operations, 11 flop.  (The column recursion it replaced takes 15, 28 flop.)
+FLOP_PER_VALUE_TUPLE = 11
+DP_OPS_PER_VALUE_TUPLE = 7
+# DRAM bytes (read + write) of one one-warp tri_walk_kernel<3,false,false,false> launch at 19456 points,
+# from one ncu capture (its output is 1.619 GB; the rest is in L2 at its end), scaled to 100000 points.
+WALK_TRAFFIC_POINTS, WALK_TRAFFIC = 19456, 1.557012224e9 + 0.217088e6
 
 
 def parse_args():
@@ -379,9 +376,9 @@ def run_ours(args) -> None:
     values_per_step = P * J * K
     value = aggregate_value(values_per_step, world, ms_per_step)
 
-    # Roofline of the walk kernel (float64-issue bound), the dominant of the step's two
-    # launches (point preparation, walk): its own device time from the timed entry point,
-    # which records CUDA events around each launch on this stream.
+    # Roofline of the walk (float64-issue bound), the step's launches: the triangle walk over the
+    # points that fill whole waves (two forms), the column walk over the rest.  Its device time comes from
+    # the timed entry point, which records CUDA events around the launches on this stream.
     import ctypes
 
     phase = (ctypes.c_float * 2)()
@@ -526,9 +523,10 @@ def run_ours(args) -> None:
                        "l2": "256 MB write between steps, outside the per-step CUDA events; each step writes 8.3 GB"},
             "roofline": {"bound": "alu", "achieved": achieved_flops / 1e12, "peak": peak_flops / 1e12,
                          "unit": "TFLOP/s", "frac": achieved_flops / peak_flops,
-                         "traffic": WALK_TRAFFIC_20000 * P / 20000 if WALK_TRAFFIC_20000 else None,
-                         "traffic_note": "ncu dram__bytes_read+write of a 20000-point launch scaled by points",
-                         "kernel": "walk_kernel<3,false,true>", "flop_per_launch": flops,
+                         "traffic": WALK_TRAFFIC * P / WALK_TRAFFIC_POINTS if WALK_TRAFFIC else None,
+                         "traffic_note": "ncu dram__bytes_read+write of a 19456-point launch scaled by points",
+                         "kernel": "tri_walk_kernel<3,false,false,true> (part waves: its one-warp form, walk_kernel)",
+                         "flop_per_launch": flops,
                          "flop_per_unit": FLOP_PER_VALUE_TUPLE, "units_per_launch": P * J,
                          "kernel_ms": kernel_ms, "point_prep_kernel_ms": statistics.mean(prep_ms),
                          "peak_source": "measured in this run: zp_probe_fp64 float64 FMA rate x 2 flop "
@@ -544,7 +542,7 @@ def run_ours(args) -> None:
             "cpu_baseline": cpu,
             "cpu_alg1_numpy": cpu_alg1,
             "clocks": clk,
-            "gpu_launches": 2 * args.steps,  # point_prep_kernel + walk_kernel per step
+            "gpu_launches": 3 * args.steps,  # tri_walk_kernel, wide and one-warp, and walk_kernel per step
             "wall_s_timed": wall,
             "extras": extras,
         }
@@ -732,26 +730,11 @@ def measure_adjoint_emulated(dev, steps: int = 2) -> dict:
     return {"workload": "series_n24", "fp64_emulated_adjoint_ms": ms_}
 
 
-def fused_fp64_ops(ns, ms) -> int:
-    """float64 operations per point of the fused kernel's walk: per column step N >= 2 the
-    recursion (2), per step with outputs the weight product (1), per output the angular product
-    (1); per column the angle addition (4)."""
-    cols = {}
-    for n, m in zip(ns, ms):
-        cols.setdefault(abs(int(m)), {}).setdefault((int(n) - abs(int(m))) // 2, 0)
-        cols[abs(int(m))][(int(n) - abs(int(m))) // 2] += 1
-    ops = 0
-    for m, steps in cols.items():
-        n_steps = max(steps) + 1
-        ops += 4 + 2 * max(0, n_steps - 2)
-        ops += sum(1 + c for c in steps.values())
-    return ops
-
-
 def measure_fused_series(dev, peaks, steps: int = 5, n_points: int = 1_000_000) -> dict:
     """The fused float64-accurate series (basis on chip, 16 sets) on the mixed_n32 points (561
     modes, 1e6 points r = sqrt(U)) against the plain float64 basis-then-DGEMM form, with the
-    fused kernel's float64 roofline (its walk issues fused_fp64_ops per point)."""
+    fused kernel's tensor rate (its digit products: per 16 modes, 9 instructions of 128 x 144 x
+    16; the kernel itself is bound by instruction issue, cutting the digits)."""
     import ctypes
 
     import numpy as np
@@ -781,9 +764,8 @@ def measure_fused_series(dev, peaks, steps: int = 5, n_points: int = 1_000_000) 
     t_fused = _events_ms(stream, lambda: run(4, out), steps)
     run(0, out64)
     t_dgemm = _events_ms(stream, lambda: run(0, out64), 2)
-    ops = fused_fp64_ops(ns, ms) * n_points
-    probe = (ctypes.c_double * 6)()
-    _lib.check("zp_probe_fp64", lib.zp_probe_fp64(0, 20000, sp, probe))
+    flops = 2 * 144 * 9 * len(ns) * n_points
+    tensor_peak = peaks.get("bf16_tflops", 1906.3) * 1e12
     diff = float((out - out64).abs().max())
     # The adjoint of the same series (grad_C, grad_r, grad_theta): the default path (grad_C by the
     # emulated GEMM, the point gradients from the fused derivative series) against the float64
@@ -812,10 +794,10 @@ def measure_fused_series(dev, peaks, steps: int = 5, n_points: int = 1_000_000) 
             "speedup_emulated_vs_dgemm_adjoint": t_adj_64 / t_adj_emu,
             "adjoint_rel_diff_vs_dgemm_gC_gr_gt": adj_diff,
             "max_abs_diff_vs_dgemm": diff, "max_abs_value": float(out64.abs().max()),
-            "roofline": {"bound": "alu", "kernel": "fused_emu_kernel (includes the coefficient digit kernels)",
-                         "fp64_ops": ops, "achieved_ops_per_s": ops / (t_fused * 1e-3),
-                         "peak_ops_per_s": probe[2], "frac": ops / (t_fused * 1e-3) / probe[2],
-                         "peak_source": "zp_probe_fp64 float64 FMA rate measured in this run"}}
+            "roofline": {"bound": "alu", "kernel": "tri_kernel (includes the coefficient digit kernels)",
+                         "issued_tensor_flop": flops, "achieved_tflops": flops / (t_fused * 1e-3) / 1e12,
+                         "peak_tflops": tensor_peak / 1e12, "frac": flops / (t_fused * 1e-3) / tensor_peak,
+                         "peak_source": "bf16 burst rate (float16 runs at the same rate)"}}
 
 
 def measure_paper_shapes(dev, steps: int = 50) -> dict:
