@@ -99,32 +99,6 @@ __device__ __forceinline__ bool mbar_wait_sleepy(uint64_t* bar, uint32_t parity,
   }
 }
 
-// mbar_wait whose polls let the hardware suspend the thread for up to about a microsecond each,
-// so that a waiting thread takes no issue slots and still wakes as soon as the phase completes.
-__device__ __forceinline__ bool mbar_wait_suspend(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                  uint64_t limit_ns = kWaitLimitNs) {
-  auto poll = [&]() {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(1000u)
-        : "memory");
-    return ok != 0;
-  };
-  if (poll()) return true;
-  const uint64_t t0 = global_timer_ns();
-  for (uint32_t i = 0;; ++i) {
-    if (poll()) return true;
-    if ((i & 15u) == 15u) {
-      if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > limit_ns) return false;
-    }
-  }
-}
-
 // Bulk copy global -> shared, completing `bytes` transaction bytes on `bar`.
 __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
   asm volatile(
