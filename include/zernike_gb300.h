@@ -355,7 +355,7 @@ ZP_API zp_status zp_batch_adjoint(zp_batch* batch, void* stream);
  * ZP_PREC_FP64_EMULATED (float64-accurate on the tensor cores, deterministic, no host
  * synchronisation): grad_theta[p] = sum_s grad_out[p][s] (dZ/dtheta C)[p][s] and grad_r likewise
  * with dZ/drho, each derivative series by the fused kernel of ZP_PREC_FP64_EMULATED's batched
- * forward (one launch each; its row sums added onto the zeroed gradients) when n_sets <= 16 and
+ * forward (one launch for both, or one each; row sums, no matrix H) when n_sets <= 16 and
  * every instance has at most 5041 modes, else by the float64 point kernel; and per instance
  * grad_coeffs = Z G by the float64-accurate GEMM of zp_series_adjoint_plan (Z walked into
  * library scratch).  Other precisions: ZP_ERR_INVALID_ARG. */

@@ -343,10 +343,10 @@ class Batch:
                   _stream(torch.device("cuda", torch.cuda.current_device())))
 
     def adjoint(self, prec: str = "fp64emu"):
-        """grad_coeffs, grad_r, grad_theta for every instance: grad_r and grad_theta by the
-        persistent float64 point kernel; grad_coeffs per instance by the float64-accurate
-        tensor-core GEMM ("fp64emu") or by the persistent float64 column kernel ("fp64", one
-        launch)."""
+        """grad_coeffs, grad_r, grad_theta for every instance.  "fp64emu": grad_r and grad_theta
+        by the fused tensor-core kernel (at most 16 sets), grad_coeffs per instance by the
+        float64-accurate tensor-core GEMM; "fp64": the persistent float64 point and column
+        kernels, one launch each."""
         code = {"fp64": 0, "fp64emu": 4}[prec]
         _lib.call("zp_batch_adjoint_prec", self.handle, code,
                   _stream(torch.device("cuda", torch.cuda.current_device())))

@@ -1,4 +1,6 @@
-// Fused float64-accurate Zernike series for up to 16 coefficient sets: the basis is built on
+// Fused float64-accurate Zernike series for up to 16 coefficient sets, the form for mode sets that
+// the triangle kernel (zp_tri.cu, 1.65 times as fast) does not take: degrees above 64, sparse or
+// duplicated sets.  The basis is built on
 // chip and fed straight to the tensor cores; no basis value, digit or partial sum is written
 // to global memory.
 //

@@ -1,4 +1,6 @@
-// The per-(point, |m|-column) recursion walk: radial polynomials, rho-derivatives, Z.
+// The per-(point, |m|-column) recursion walk: radial polynomials, rho-derivatives, Z, for calls
+// or points that the triangle walk (zp_tri_walk.cu) does not take: few points, sparse or duplicated
+// sets, Z without derivatives, the last part of a wave.
 //
 // Work decomposition (Algorithm 1 of Sec. 3, mapped to the GPU): one thread owns
 // one or two consecutive points of one |m| column and walks the Jacobi degree N = 0 .. N_max in
