@@ -430,6 +430,7 @@ struct zp_batch {
   // The triangle form of the same launches, when every instance's plan has that layout: descriptors
   // of the values, then of the gradients, sharing items, digits and scales.
   bool tri_ok = false;
+  bool point_grads = false;  // some instance with modes and points wants grad_r or grad_theta
   void* tri_block = nullptr;
   zp::TriInst* d_tinst = nullptr;
   int32_t* d_tchunk = nullptr;
@@ -633,13 +634,12 @@ zp_status build_fused(zp_batch* b) {
 zp_status build_tri(zp_batch* b) {
   if (!b->fused_ok) return ZP_OK;
   const int64_t n = (int64_t)b->inst.size();
-  bool grads = false;
+  const bool grads = b->point_grads;
   for (int64_t i = 0; i < n; ++i) {
     if (b->inst[i].n_modes == 0) continue;
     const zp_plan* p = b->plans[b->inst_plan[i]].get();
     if (!p->tri) return ZP_OK;
     b->tri_n_max = std::max(b->tri_n_max, p->n_max);
-    grads |= b->inst[i].grad_r || b->inst[i].grad_theta;
   }
   std::vector<TriInst> ti(2 * n);
   std::vector<int32_t> chunk_inst;
@@ -761,6 +761,7 @@ zp_status zp_batch_create(const zp_instance* instances, int64_t n_instances, int
   for (int64_t i = 0; i < n_instances; ++i) {
     const zp_instance& in = b->inst[i];
     ZP_TRY(batch_validate_ptrs(in, n_sets, i));
+    b->point_grads |= in.n_modes > 0 && in.n_points > 0 && (in.grad_r || in.grad_theta);
     if (in.n_modes > 0 && (!in.n || !in.m)) return set_error(ZP_ERR_INVALID_ARG, "instance mode list is NULL");
     auto key = std::make_pair(std::vector<int32_t>(in.n, in.n + in.n_modes), std::vector<int32_t>(in.m, in.m + in.n_modes));
     auto it = seen.find(key);
@@ -941,12 +942,14 @@ static zp_status zp_batch_adjoint_impl(zp_batch* b, zp_precision prec, void* str
   if (prec != ZP_PREC_FP64 && prec != ZP_PREC_FP64_EMULATED)
     return set_error(ZP_ERR_INVALID_ARG, "batched adjoint supports ZP_PREC_FP64 and ZP_PREC_FP64_EMULATED");
   cudaStream_t st = (cudaStream_t)stream;
-  bool need_pt = false, need_c = false;
+  // Instances without modes or points take no launch: the buffers of the gradient form exist only when
+  // one with both asks for a point gradient.
+  const bool need_pt = b->point_grads;
+  bool need_c = false;
   for (size_t i = 0; i < b->inst.size(); ++i) {
     const zp_instance& in = b->inst[i];
     if (in.n_points > 0 && in.n_modes > 0 && b->n_sets > 0 && !in.grad_out)
       return set_error(ZP_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": grad_out is NULL");
-    need_pt |= in.grad_r || in.grad_theta;
     need_c |= in.grad_coeffs != nullptr;
   }
   // Instances with no modes or no points: zero what exists (empty sums).
