@@ -115,14 +115,16 @@ __device__ __forceinline__ double pivot_reciprocal(double v) {
 
 // Panel k0 (columns k0 .. k0 + nb - 1, the updates of earlier panels already applied): every
 // CTA factors the nb x nb diagonal block in shared memory (identical arithmetic, so the copies
-// agree bitwise); CTA 0 writes the factor back, CTA b >= 1 solves rows k0 + 32 b ... of the
-// panel against it (L_rows = A_rows L_kk^-T).  info[0]: 1 + the first column whose pivot is not
-// positive (left 0 when there is none).
+// agree bitwise); CTA 0 writes the factor out, CTA b >= 1 solves rows k0 + 32 b ... of the
+// panel against it (L_rows = A_rows L_kk^-T).  CTA 0 leaves A's diagonal block alone while other CTAs
+// may still have to read it (they need not all be resident at once): its factor goes to `diag` [32][32]
+// and the update launch that follows stores it in A; the last panel, one CTA, writes A itself.
+// info[0]: 1 + the first column whose pivot is not positive (left 0 when there is none).
 // Bound: the chain of 32 pivots.  The columns stay unscaled during the elimination (a_rq -= a_rc
 // a_qc / v_c), so a pivot costs one reciprocal, taken by the thread that has just formed it, and one
 // barrier instead of a square root and three; the square roots come at the end, all at once.  Below
 // the block eight threads share a row (four columns each).  48.6 -> 30.4 us per panel.
-__global__ void __launch_bounds__(256) chol_panel_kernel(double* A, int J, int k0, int* info) {
+__global__ void __launch_bounds__(256) chol_panel_kernel(double* A, int J, int k0, double* diag, int* info) {
   __shared__ double D[kNb][kNb + 1];  // unscaled columns: D[r][c], r >= c, pivots on the diagonal
   __shared__ double R[kNb][kNb + 1];
   __shared__ double r2[kNb], rd[kNb], dg[kNb];
@@ -164,8 +166,11 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(double* A, int J, int k
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int c = ty + 8 * i;
-      if (tx < nb && c < nb && tx >= c)
-        A[(size_t)(k0 + tx) + (size_t)(k0 + c) * J] = tx == c ? dg[c] : D[tx][c] * rd[c];
+      if (tx < nb && c < nb && tx >= c) {
+        const double l = tx == c ? dg[c] : D[tx][c] * rd[c];
+        if (gridDim.x == 1) A[(size_t)(k0 + tx) + (size_t)(k0 + c) * J] = l;
+        else diag[c * kNb + tx] = l;
+      }
     }
     return;
   }
@@ -188,8 +193,9 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(double* A, int J, int k
 }
 
 // Trailing update after panel k0: A[i][j] -= sum_u L[i][k0+u] L[j][k0+u] for k0 + 32 <= j <= i,
-// one 32 x 32 tile (tile row ti >= tile column tj) per CTA, 4 outputs per thread.
-__global__ void __launch_bounds__(256) chol_update_kernel(double* A, int J, int k0) {
+// one 32 x 32 tile (tile row ti >= tile column tj) per CTA, 4 outputs per thread.  The last CTA also
+// stores the panel's factored diagonal block, which no CTA of this launch reads from A.
+__global__ void __launch_bounds__(256) chol_update_kernel(double* A, int J, int k0, const double* diag) {
   __shared__ double Li[kNb][kNb + 1], Lj[kNb][kNb + 1];
   const int k1 = k0 + kNb;
   const int t = (int)blockIdx.x;
@@ -199,6 +205,10 @@ __global__ void __launch_bounds__(256) chol_update_kernel(double* A, int J, int 
   const int i0 = k1 + ti * kNb, j0 = k1 + tj * kNb;
   const int ri = min(kNb, J - i0), rj = min(kNb, J - j0);
   const int tid = threadIdx.x;
+  for (int e = tid; blockIdx.x == gridDim.x - 1 && e < kNb * kNb; e += blockDim.x) {
+    const int r = e % kNb, c = e / kNb;
+    if (r >= c) A[(size_t)(k0 + r) + (size_t)(k0 + c) * J] = diag[e];
+  }
   for (int e = tid; e < kNb * kNb; e += blockDim.x) {
     const int r = e % kNb, c = e / kNb;
     Li[r][c] = r < ri ? A[(size_t)(i0 + r) + (size_t)(k0 + c) * J] : 0.0;
@@ -401,17 +411,17 @@ __global__ void __launch_bounds__(256) trsm_update_kernel(const double* __restri
 }
 
 // Right-looking blocked Cholesky factorisation of the J x J normal matrix in place (lower
-// triangle, column-major); info[0] as in chol_panel_kernel (zeroed here).
-zp_status cholesky_factor(double* A, int J, int* info, cudaStream_t stream) {
+// triangle, column-major); info[0] as in chol_panel_kernel (zeroed here).  diag: kNb * kNb scratch.
+zp_status cholesky_factor(double* A, int J, double* diag, int* info, cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(info, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
   for (int k0 = 0; k0 < J; k0 += kNb) {
     const int nb = std::min(kNb, J - k0);
     const int below = J - k0 - nb;
-    chol_panel_kernel<<<1 + (below + kNb - 1) / kNb, 256, 0, stream>>>(A, J, k0, info);
+    chol_panel_kernel<<<1 + (below + kNb - 1) / kNb, 256, 0, stream>>>(A, J, k0, diag, info);
     if (below > 0) {
       const int64_t nt = (below + kNb - 1) / kNb;
-      chol_update_kernel<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, stream>>>(A, J, k0);
+      chol_update_kernel<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, stream>>>(A, J, k0, diag);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "Cholesky panel launch");
   }
@@ -424,9 +434,10 @@ zp_status blocked_cholesky_solve(const double* A, int J, double* B, int S, doubl
 
 // Factors the J x J normal matrix (J <= kCholMaxJ) in place and solves for the J x S
 // right-hand sides B (column-major), storing the solution row-major [J][S] in X; info[0] as in
-// chol_panel_kernel (zeroed here).
-zp_status small_cholesky_solve(double* A, int J, const double* B, int S, double* X, int* info, cudaStream_t stream) {
-  ZP_TRY(cholesky_factor(A, J, info, stream));
+// chol_panel_kernel (zeroed here), diag as in cholesky_factor.
+zp_status small_cholesky_solve(double* A, int J, const double* B, int S, double* X, double* diag, int* info,
+                               cudaStream_t stream) {
+  ZP_TRY(cholesky_factor(A, J, diag, info, stream));
   cudaError_t e;
   static DeviceMemo<int> attr;  // the solve's shared memory limit, set once per device
   int limit = 0;
@@ -515,7 +526,8 @@ zp_status series_fit_fp64(const zp_plan* plan, const double* r, const double* th
   ZP_TRY(zbuf.alloc((size_t)J * P * sizeof(double), stream));
   ZP_TRY(gram.alloc((size_t)J * J * sizeof(double), stream));
   ZP_TRY(rhs.alloc((size_t)J * S * sizeof(double), stream));
-  ZP_TRY(info.alloc(4 * sizeof(double), stream));  // [0]: potrf status (int), [2..3]: pivot range
+  // [0]: potrf status (int), [2..3]: pivot range, [4..]: a panel's diagonal block
+  ZP_TRY(info.alloc((4 + kNb * kNb) * sizeof(double), stream));
   double* Z = (double*)zbuf.ptr;
   ZP_TRY(launch_walk(plan, r, theta, P, 0, Z, nullptr, stream));
   const double* Yuse = Y;
@@ -553,10 +565,10 @@ zp_status series_fit_fp64(const zp_plan* plan, const double* r, const double* th
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "add_ridge_kernel launch");
   }
   if (J <= kCholMaxJ) {
-    ZP_TRY(small_cholesky_solve((double*)gram.ptr, (int)J, (const double*)rhs.ptr, (int)S, coeffs, (int*)info.ptr,
-                                stream));
+    ZP_TRY(small_cholesky_solve((double*)gram.ptr, (int)J, (const double*)rhs.ptr, (int)S, coeffs, (double*)info.ptr + 4,
+                                (int*)info.ptr, stream));
   } else {
-    ZP_TRY(cholesky_factor((double*)gram.ptr, (int)J, (int*)info.ptr, stream));
+    ZP_TRY(cholesky_factor((double*)gram.ptr, (int)J, (double*)info.ptr + 4, (int*)info.ptr, stream));
     ZP_TRY(blocked_cholesky_solve((const double*)gram.ptr, (int)J, (double*)rhs.ptr, (int)S, coeffs, stream));
   }
   pivot_range_kernel<<<1, 256, 0, stream>>>((const double*)gram.ptr, J, (double*)info.ptr + 2);
