@@ -978,6 +978,7 @@ __global__ void __launch_bounds__(gemm_threads<CG>(), 1) split_gemm_kernel(GemmA
               if (cbase + i < cend) frow[cbase + i] = __uint_as_float(v[i]);
           }
         }
+        __syncwarp();  // the next tensor-memory load is the whole warp's
       }
       // The warp's loads of this accumulator are done: one arrive per warp (remote for the odd
       // CTA of a pair, whose accumulators the even CTA's MMAs fill).
@@ -1202,6 +1203,7 @@ __global__ void __launch_bounds__(192, 1) stacked_slice_gemm_kernel(StackedArgs 
             for (int i = 0; i < (int)a.N; ++i) dst[i] = x[i];
           }
         }
+        __syncwarp();  // the next tensor-memory load is the whole warp's
       }
       ptx::tc_fence_before();
       __syncwarp();

@@ -246,24 +246,28 @@ __device__ __forceinline__ bool drain_segment(const TriArgs& a, const Pending& p
         else lo[i] = horner(lo[i], 6, tv);
       }
     }
-    if (p >= d.P) continue;
     const int e_base = pd.ep - 6 * (TND + 1);
     const int* cexp = d.cexp + g * TNS;
+    if (p < d.P) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int s = half * 8 + i;
-      if (s >= d.S) break;
-      const int ec = cexp[s];
-      const double v = (pd.ep == kNonFiniteRow || ec == kNonFiniteRow)
-                           ? __longlong_as_double(0x7ff8000000000000ll)
-                           : join_rounded(hi[i], lo[i], 6 * (TND - Split), e_base + ec);
-      if constexpr (GROUPS == 2) {
-        dot[g] = fma(d.gdot[p * d.S + s], v, dot[g]);
-      } else {
-        double* o = d.out + p * d.S + s;
-        *o = pd.first ? v : *o + v;
+      for (int i = 0; i < 8; ++i) {
+        const int s = half * 8 + i;
+        if (s >= d.S) break;
+        const int ec = cexp[s];
+        const double v = (pd.ep == kNonFiniteRow || ec == kNonFiniteRow)
+                             ? __longlong_as_double(0x7ff8000000000000ll)
+                             : join_rounded(hi[i], lo[i], 6 * (TND - Split), e_base + ec);
+        if constexpr (GROUPS == 2) {
+          dot[g] = fma(d.gdot[p * d.S + s], v, dot[g]);
+        } else {
+          double* o = d.out + p * d.S + s;
+          *o = pd.first ? v : *o + v;
+        }
       }
     }
+    // All lanes take the next tensor-memory load together: those beyond the last point, and those that
+    // join_rounded parted, meet here.
+    __syncwarp();
   }
   if constexpr (GROUPS == 2) {
     // The two halves' sums of a point meet in shared memory.
@@ -580,6 +584,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
                 digits_of(y[0], y[1], w[2 * h], dc);
                 digits_of(y[2], y[3], w[2 * h + 1], dc);
               }
+              __syncwarp();  // to_fixed parts the lanes; a tensor-memory store is the whole warp's
               store_digits(lane_base + (uint32_t)stage * kAStage + 4u * k, w[0], w[1], w[2], w[3]);
               bi.advance(H);
             }
