@@ -18,7 +18,7 @@
 // keeps the pipe two thirds busy: the instructions between two float64 operations are not hidden.
 // The wide form (radial, k >= 2) holds the row's two highest derivative lanes in tensor memory (each
 // warp reads its own 32 lanes of it), so that two warps per scheduler fit: eight in a block, one
-// block per SM.  The next block's lanes are read under the operations of this one.
+// block per SM.
 //
 // Measured against the column form: radial set n <= 100, k <= 3, 1e5 points 6.32 -> 3.66 ms (4.62
 // with one warp per scheduler); Z and dZ/drho with dZ/dtheta, n <= 32, 99991 points 836 -> 631 us.
@@ -154,37 +154,42 @@ __global__ void __launch_bounds__(WIDE ? kWideWarps * W : W) tri_walk_kernel(Tri
 #pragma unroll
     for (int k = 0; k < L; ++k) l0[k] = l1[k] = dg[k] = 0.0;
     if (A == 0) dg[0] = -1.0;
-    uint32_t v[8] = {};  // the row above in tensor memory
-    if constexpr (WIDE) {
-      if (A > 0) ptx::tmem_ld_32x32b_x8(tm, v);
-    }
 #pragma unroll kUnroll
     for (int B = 0; B <= nb; ++B, ++block) {
-      if constexpr (WIDE) __syncwarp();
+      // The row above.  Its lanes in tensor memory arrive asynchronously: loaded for every block (also
+      // those that do not use them, whose columns are the block's own) and waited for in the same
+      // straight-line stretch, so that nothing can touch the registers in between.
+      uint32_t v[8];
+      if constexpr (WIDE) {
+        __syncwarp();
+        ptx::tmem_ld_32x32b_x8(tm + 8 * B, v);
+      }
       const int4 jc = __ldg(perm + 2 * block), js = __ldg(perm + 2 * block + 1);
       double* row = st + (size_t)(2 * B) * LS * W;
       double u0[L], u1[L], e00[L], e01[L], e10[L], e11[L];
-#pragma unroll
-      for (int k = 0; k < LS; ++k) {
-        u0[k] = B < A ? row[k * W] : l0[k];
-        u1[k] = B < A ? row[(LS + k) * W] : l1[k];
-      }
       if constexpr (WIDE) {
-        if (B < A) {
-          ptx::tmem_ld_wait(v);
 #pragma unroll
-          for (int k = 0; k < kWideLanes; ++k) {
-            u0[LS + k] = __hiloint2double((int)v[2 * k + 1], (int)v[2 * k]);
-            u1[LS + k] = __hiloint2double((int)v[2 * k + 5], (int)v[2 * k + 4]);
-          }
-        } else {
-#pragma unroll
-          for (int k = LS; k < L; ++k) {
-            u0[k] = l0[k];
-            u1[k] = l1[k];
-          }
+        for (int k = 0; k < LS; ++k) {
+          u0[k] = row[k * W];
+          u1[k] = row[(LS + k) * W];
         }
-        if (B + 1 < A && B < nb) ptx::tmem_ld_32x32b_x8(tm + 8 * B + 8, v);  // the next block's, under this one's operations
+        ptx::tmem_ld_wait(v);
+#pragma unroll
+        for (int k = 0; k < kWideLanes; ++k) {
+          u0[LS + k] = __hiloint2double((int)v[2 * k + 1], (int)v[2 * k]);
+          u1[LS + k] = __hiloint2double((int)v[2 * k + 5], (int)v[2 * k + 4]);
+        }
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+          u0[k] = B < A ? u0[k] : l0[k];
+          u1[k] = B < A ? u1[k] : l1[k];
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+          u0[k] = B < A ? row[k * W] : l0[k];
+          u1[k] = B < A ? row[(L + k) * W] : l1[k];
+        }
       }
       const int n0 = 2 * (A + B), m0 = 2 * (A - B);
       const double nd0 = num[n0], nd1 = num[n0 + 1], nd2 = num[n0 + 2];
