@@ -68,9 +68,10 @@ typedef enum {
   ZP_PREC_FP64 = 0,   /* the plain float64 basis-then-GEMM form, kept as the baseline: the basis
                          is written to scratch and contracted by cuBLAS DGEMM; outputs float64.
                          The library's default float64 path is ZP_PREC_FP64_EMULATED */
-  ZP_PREC_BF16X3 = 1, /* float64 basis, contraction on tensor cores as hi*hi + hi*lo + lo*hi
+  ZP_PREC_BF16X3 = 1, /* basis in float64 or, for filled triangles n <= 71, in pairs of float32 (45 bits of
+                         each value), contraction on tensor cores as hi*hi + hi*lo + lo*hi
                          with bfloat16 halves and float32 accumulation; outputs float32 */
-  ZP_PREC_TF32 = 2,   /* float64 basis rounded to TF32, tensor-core contraction with float32
+  ZP_PREC_TF32 = 2,   /* the same basis rounded to TF32, tensor-core contraction with float32
                          accumulation; outputs float32 */
   ZP_PREC_FP32 = 3,   /* float64 basis rounded to float32, float32 contraction on the CUDA
                          cores; outputs float32 (batched forward only) */
@@ -171,7 +172,7 @@ ZP_API zp_status zp_radial_per_mode(const zp_plan* plan, const double* r, int64_
  * ZP_PREC_FP64_EMULATED is the float64-accurate form to use; ZP_PREC_FP64 is the plain
  * baseline: it writes the basis to scratch device memory (allocated stream-ordered on `stream`
  * from the library's scratch pool, see zp_release_scratch, and released to it before return)
- * and contracts with cuBLAS DGEMM.  The split forms run the float64 recursion into
+ * and contracts with cuBLAS DGEMM.  The split forms run the recursion into
  * tensor-core operand tiles in scratch (slabs of whole waves of point tiles) and contract them
  * with tcgen05 MMAs and float32 accumulation.  ZP_PREC_FP64_EMULATED with n_sets <= 16 and at
  * most 5041 padded modes builds the basis inside the tensor-core kernel (no basis in memory):

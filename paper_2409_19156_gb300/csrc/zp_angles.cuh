@@ -16,23 +16,37 @@ __device__ __forceinline__ double from_fixed62(int64_t v) {
   return __longlong_as_double((long long)(b | ((uint64_t)v & (1ull << 63))));
 }
 
-// Calls f(m, cos m theta, sin m theta) for m = 0 .. m_max.  In fixed point (absolute errors below 2^-57;
+// The same as a float32 (24 bits of the larger part).
+__device__ __forceinline__ float from_split62(const TriTrig& t) { return fmaf((float)t.lo, 0x1p-62f, (float)t.hi * 0x1p-31f); }
+
+// Calls f(m, cos m theta, sin m theta) for m = 0 .. m_max, in T.  In fixed point (absolute errors below 2^-57;
 // a float64 product m theta alone rounds by up to 2^-53 m theta) unless the angle is so small that
 // sin(m theta) needs relative accuracy, or out of range: then by angle addition in float64, restarted
-// from sincos at every 16th m.
-template <typename F>
+// from sincos at every 16th m.  (For float32 results fixed point serves as long as neither cos theta
+// nor sin theta is below 2^-36: 26 bits of either are left.)
+template <typename T = double, typename F>
 __device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
+  constexpr bool kFloat = sizeof(T) == sizeof(float);
   const double mag = fabs(th);
-  if (mag >= 1.0 / 128 && mag < 2048.0) {
-    int64_t ci, si;
+  int64_t ci = 0, si = 0;
+  bool fixed = mag < 2048.0 && (kFloat || mag >= 1.0 / 128);
+  if (fixed) {
     tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
+    if constexpr (kFloat) fixed = min(llabs(ci), llabs(si)) >= 1ll << 26;
+  }
+  if (fixed) {
     const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
     TriTrig c = tri_split(1ll << 62), s = tri_split(0);
-    f(0, 1.0, 0.0);
+    f(0, T(1), T(0));
     for (int m = 1; m <= m_max; ++m) {
       tri_rotate(c, s, c1, s1);
-      f(m, from_fixed62((int64_t)c.hi * (1ll << 31) + c.lo), from_fixed62((int64_t)s.hi * (1ll << 31) + s.lo));
+      if constexpr (kFloat)
+        f(m, from_split62(c), from_split62(s));
+      else
+        f(m, from_fixed62((int64_t)c.hi * (1ll << 31) + c.lo), from_fixed62((int64_t)s.hi * (1ll << 31) + s.lo));
     }
+  } else if (kFloat && th == 0.0) {
+    for (int m = 0; m <= m_max; ++m) f(m, T(1), T(0));
   } else {
     double s1, c1, c = 1.0, s = 0.0;
     sincos(th, &s1, &c1);
@@ -44,7 +58,7 @@ __device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
         s = fma(s, c1, c * s1);
         c = cn;
       }
-      f(m, c, s);
+      f(m, T(c), T(s));
     }
   }
 }

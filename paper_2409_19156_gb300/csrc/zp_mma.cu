@@ -35,9 +35,11 @@
 #include "zp_device.cuh"
 #include "zp_api_common.h"
 #include "zp_ptx.cuh"
+#include "zp_angles.cuh"
 #include "zp_emu_device.cuh"
 #include "zp_emu_shape.h"
 #include "zp_fused.h"
+#include "zp_pair.h"
 #include "zp_tri_host.h"
 #include "zp_series_internal.h"
 
@@ -347,13 +349,18 @@ __device__ __forceinline__ void split_basis_tile(const BasisArgs& a, int64_t til
 }
 
 // ---------------------------------------------------------------------------------------
-// The same operand from the fixed-point triangle walk (zp_tri.h), for mode lists that have its
-// layout.  The float64 recursion above holds the float64 pipe for two operations per (n, |m|) and
-// point; here the walk runs on the integer pipe in 64-bit fixed point, the values become float32
-// from their upper 32 bits (2^-31 absolute; the operands keep 16 or 11 significant bits of their
-// own) and the angular products stay float32.  K order: first the blocks whose eight elements
-// (four cos, four sin) all have modes, eight positions each, so that a block is a whole 16-byte unit
-// per operand part with no packing across blocks; then the other blocks' modes one by one.
+// The same operand from the walk over a filled triangle (zp_tri.h has the recursion and the layout).
+// The float64 recursion above holds the float64 pipe for two operations per (n, |m|) and point; here a
+// value is an unevaluated sum of two float32 (zp_pair.h), about 45 bits relative to itself, of
+// which the operands keep 16 or 11: small values near the origin stay as accurate as large ones.
+// Angles come from the fixed-point functions (zp_angles.cuh).  No point takes another path.  K order:
+// first the blocks whose eight elements (four cos, four sin) all have modes, eight positions each, so
+// that a block is a whole 16-byte unit per operand part with no packing across blocks; then the other
+// blocks' modes one by one.
+// Bound: instruction issue.  n <= 32, 2e5 points: 153-164 us, against 381 us by columns in float64 and
+// 310-319 us with this walk in float64 (its own pipe is then the bound); n <= 27, 150001 points, TF32:
+// 102, 185 and 195 us.  (Radial words of 64-bit fixed point cut to 31 bits and angles of 32 bits took
+// 129 and 86 us, and lost every digit of values below 1e-9.)
 struct TriBasisArgs {
   const int32_t* perm;  // modes of the triangle's positions, -1 for none
   const double* r;
@@ -372,45 +379,18 @@ __host__ __device__ constexpr uint32_t tri_basis_smem(int n_max) {
 // Two blocks or more per SM.
 constexpr uint32_t kTriBasisSmem = 110 * 1024;
 
-// cos and sin of a fraction of a turn (its upper 32 bits) to float32 accuracy: the nearest quarter turn
-// taken off, Taylor polynomials of the rest.  A third of the fixed-point rotation's instructions,
-// and every multiple of the angle is evaluated by itself.
-__device__ __forceinline__ float2 turn_cos_sin(uint32_t turn) {
-  const uint32_t k = (turn + 0x20000000u) >> 30;
-  const float x = (float)(int32_t)(turn - (k << 30)) * 1.4629180792671596e-9f;  // 2 pi / 2^32
-  const float u = x * x;
-  const float s = fmaf(x * u, fmaf(u, fmaf(u, fmaf(u, 1.0f / 362880, -1.0f / 5040), 1.0f / 120), -1.0f / 6), x);
-  const float c = fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.0f / 40320, -1.0f / 720), 1.0f / 24), -0.5f), 1.0f);
-  const float a = (k & 1u) ? s : c, b = (k & 1u) ? c : s;
-  return make_float2(__uint_as_float(__float_as_uint(a) ^ (((k + 1u) & 2u) << 30)),
-                     __uint_as_float(__float_as_uint(b) ^ ((k & 2u) << 30)));
-}
-
-template <bool TF32, bool SLOW>
+template <bool TF32>
 __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA, uint32_t row, double rho, double th,
-                                              uint64_t* st, float2* an, const uint8_t* whole) {
+                                              float2* st, float2* an, const uint8_t* whole) {
   using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
   constexpr int UNIT = TF32 ? 4 : 8;
   const int n_max = a.n_max, H = n_max / 2;
-  TriPoint tp = {};
-  if constexpr (!SLOW) {
-    tp = tri_point((uint64_t)__double_as_longlong(rho));
-    const uint64_t turn = tri_turn((uint64_t)__double_as_longlong(th));
-    uint64_t t = 1ull << 31;
-    for (int m = 0; m <= n_max; ++m, t += turn) {
-      const float2 g = turn_cos_sin((uint32_t)(t >> 32));
-      an[(size_t)m * BM] = make_float2(g.x * 0x1p-30f, g.y * 0x1p-30f);  // the radial word's 2^-30
-    }
-  } else {
-    double s1, c1, c = 1.0, s = 0.0;
-    sincos(th, &s1, &c1);
-    for (int m = 0; m <= n_max; ++m) {
-      an[(size_t)m * BM] = make_float2(float_of_double(c), float_of_double(s));
-      const double cn = fma(c, c1, -s * s1);
-      s = fma(s, c1, c * s1);
-      c = cn;
-    }
-  }
+  // (A constant needs no radius, and takes none that is not finite.)
+  rho = n_max > 0 ? rho : 0.0;
+  for_each_angle<float>(th, n_max, [&](int m, float c, float s) { an[(size_t)m * BM] = make_float2(c, s); });
+  const float rh = (float)rho, rl = isfinite(rh) ? (float)(rho - (double)rh) : 0.0f;
+  const PairFactor<float> r1{rh, -rh, -rl};
+  const PairFactor<f32x2> r2{f32x2::of(rh, rh), f32x2::of(-rh, -rh), f32x2::of(-rl, -rl)};
   int k_full = 0, k_tail = 8 * a.full;
   Pack16 hi, lo;
   auto at = [&](int k, uint32_t r) {  // a unit's place in row r
@@ -453,42 +433,20 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
   int block = 0;
   for (int A = 0; A <= H; ++A) {
     const int nb = min(A, H - A);
-    uint64_t l0 = SLOW ? 0ull : kTriZero, l1 = l0;
-    uint64_t dg = A == 0 ? (SLOW ? (uint64_t)__double_as_longlong(-1.0) : 0ull) : l0;
+    float2 l0 = make_float2(0.0f, 0.0f), l1 = l0, dg = make_float2(A == 0 ? -1.0f : 0.0f, 0.0f);
     for (int B = 0; B <= nb; ++B, ++block) {
-      uint64_t* sr = st + (size_t)(2 * B) * BM;
-      const uint64_t u0 = B < A ? sr[0] : l0, u1 = B < A ? sr[BM] : l1;
-      uint64_t e00, e01, e10, e11;
-      float f[4];
-      if constexpr (!SLOW) {
-        e00 = tri_step(tp, u0, l0, dg);
-        e01 = tri_step(tp, u1, e00, u0);
-        e10 = tri_step(tp, e00, l1, l0);
-        e11 = tri_step(tp, e01, e10, e00);
-        auto upper = [](uint64_t e) { return (float)(int32_t)((uint32_t)(e >> 31) - (1u << 30)); };
-        f[0] = upper(e00);
-        f[1] = upper(e01);
-        f[2] = upper(e10);
-        f[3] = upper(e11);
-      } else {
-        auto d = [](uint64_t v) { return __longlong_as_double((long long)v); };
-        auto w = [](double v) { return (uint64_t)__double_as_longlong(v); };
-        const double x00 = fma(rho, d(u0) + d(l0), -d(dg)), x01 = fma(rho, d(u1) + x00, -d(u0));
-        const double x10 = fma(rho, x00 + d(l1), -d(l0)), x11 = fma(rho, x01 + x10, -x00);
-        e00 = w(x00);
-        e01 = w(x01);
-        e10 = w(x10);
-        e11 = w(x11);
-        f[0] = float_of_double(x00);
-        f[1] = float_of_double(x01);
-        f[2] = float_of_double(x10);
-        f[3] = float_of_double(x11);
-      }
+      float2* sr = st + (size_t)(2 * B) * BM;
+      const float2 u0 = B < A ? sr[0] : l0, u1 = B < A ? sr[BM] : l1;
+      const float2 e00 = pair_step(r1, u0, l0, dg);
+      float2 e01, e10;  // independent of each other: one instruction for both
+      pair_step2(r2, u1, e00, u0, e00, l1, l0, e01, e10);
+      const float2 e11 = pair_step(r1, e01, e10, e00);
       sr[0] = e10;
       sr[BM] = e11;
       dg = u1;
       l0 = e01;
       l1 = e11;
+      const float f[4] = {e00.x + e00.y, e01.x + e01.y, e10.x + e10.y, e11.x + e11.y};
       const int m0 = 2 * (A - B);
       const float2 mid = an[(size_t)m0 * BM], low = an[(size_t)max(m0 - 1, 0) * BM], top = an[(size_t)min(m0 + 1, n_max) * BM];
       const float z[8] = {f[0] * mid.x, f[1] * low.x, f[2] * top.x, f[3] * mid.x,
@@ -540,9 +498,9 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
 template <bool TF32>
 __global__ void __launch_bounds__(BM) tri_basis_kernel(TriBasisArgs a) {
   using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
-  extern __shared__ uint64_t tri_basis_mem[];
-  uint64_t* st = tri_basis_mem + threadIdx.x;
-  float2* angles = reinterpret_cast<float2*>(tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM);
+  extern __shared__ float2 tri_basis_mem[];
+  float2* st = tri_basis_mem + threadIdx.x;
+  float2* angles = tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM;
   float2* an = angles + threadIdx.x;
   // Which blocks have all their modes (a load per block would stall on its latency).
   uint8_t* whole = reinterpret_cast<uint8_t*>(angles + (size_t)(a.n_max + 1) * BM);
@@ -554,12 +512,8 @@ __global__ void __launch_bounds__(BM) tri_basis_kernel(TriBasisArgs a) {
   const int64_t p = (a.mt_base + blockIdx.x) * BM + threadIdx.x;
   const bool valid = p < a.P;
   const double rho = valid ? a.r[p] : 0.0, th = valid ? a.theta[p] : 0.0;
-  const uint32_t e = ((uint32_t)__double2hiint(th) >> 20) & 0x7ffu;
   uint8_t* gA = a.A + (size_t)blockIdx.x * a.KC * C::A_CHUNK;
-  if (__any_sync(0xffffffffu, !(rho >= 0.0 && rho <= 1.0 && e < (uint32_t)kTriAngleExponent)))
-    tri_basis_row<TF32, true>(a, gA, threadIdx.x, rho, th, st, an, whole);
-  else
-    tri_basis_row<TF32, false>(a, gA, threadIdx.x, rho, th, st, an, whole);
+  tri_basis_row<TF32>(a, gA, threadIdx.x, rho, th, st, an, whole);
 }
 
 struct CoeffArgs {
