@@ -31,9 +31,10 @@ constexpr int kTriMaxWalkN = 256; // largest n_max of the float64 walk over the 
 constexpr int kTriDigits = 9;     // base-64 digits per value
 constexpr int kTriChunk = 16;     // positions per chunk (one tensor-core K step)
 // Longest run of positions whose diagonal sums stay below 2^24 (exact in float32): digits of at
-// most 33 (values) and 65 (coefficients) in front, 32 behind, so a position adds at most
-// 33 * 32 + 65 * 32 + 7 * 32^2 = 10304 to the largest kept diagonal.
-constexpr int kTriMaxRun = 1600;  // positions: 1600 * 10304 < 2^24
+// most 63 (values; 33 on the disc, but a row off it is scaled to just below twice that) and 65
+// (coefficients) in front, 32 behind, so a position adds at most 63 * 32 + 65 * 32 + 7 * 32^2 = 11264 to
+// the largest kept diagonal.
+constexpr int kTriMaxRun = 1489;  // positions: 1489 * 11264 < 2^24
 
 // The number of blocks in rows before A, and in all rows, of the triangle with H = n_max / 2.
 __host__ __device__ constexpr int tri_blocks_before(int A, int H) {
