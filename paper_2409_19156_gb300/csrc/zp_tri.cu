@@ -843,6 +843,21 @@ __global__ void __launch_bounds__(kTriChunk * TNS) tri_deriv_kernel(TriArgs a, c
   const int pos = (int)kc * kTriChunk + threadIdx.x / TNS;
   int n, m, sine;
   tri_mode(pos, d.n_max, n, m, sine);
+  // A set with coefficients near the top of the range is formed 2^-24 down (the sums below grow by at most
+  // (n + 1) 96 < 2^13), which its scale takes up again.
+  __shared__ int high[TNS];
+  if (threadIdx.x < TNS) high[threadIdx.x] = 0;
+  __syncthreads();
+  if (s < d.S) {
+    bool top = false;
+#pragma unroll 8
+    for (int64_t j = threadIdx.x / TNS; j < d.J; j += kTriChunk) top |= !(fabs(d.coeffs[j * d.S + s]) < 0x1p1000);
+    if (top) high[s] = 1;
+  }
+  __syncthreads();
+  const int down = high[s] ? 24 : 0;
+  const double scale = down ? 0x1p-24 : 1.0;
+  if (kc == 0 && threadIdx.x < TNS) d.cexp[s] = d.cexp[TNS + s] = down;  // tri_coeff_kernel adds the rest
   double vx = 0.0, vy = 0.0;
   if (s < d.S && m >= 0 && n < d.n_max && !(m == 0 && sine)) {
     // Sums over n' = n + 1, n + 3, .. of the coefficients of (n', mm), cos or sin.
@@ -852,7 +867,7 @@ __global__ void __launch_bounds__(kTriChunk * TNS) tri_deriv_kernel(TriArgs a, c
       for (int k = n + 1; k <= d.n_max; k += 2) {
         if (mm > k) continue;
         const int32_t j = __ldg(d.perm + tri_position(k, mm, h, d.n_max));
-        if (j >= 0) t += d.coeffs[(int64_t)j * d.S + s];
+        if (j >= 0) t = fma(scale, d.coeffs[(int64_t)j * d.S + s], t);
       }
       return t;
     };
@@ -871,7 +886,8 @@ __global__ void __launch_bounds__(kTriChunk * TNS) tri_deriv_kernel(TriArgs a, c
 }
 
 // Coefficient digits of one chunk and group (blockIdx.y): the sets' scales 2^e > max |C| (formed by
-// every block from all of the group's coefficients; the first chunk's block stores them), then
+// every block from all of the group's coefficients; the first chunk's block stores them, with what
+// tri_deriv_kernel took off), then
 // 9 digits per coefficient as float16 rows of 32 bytes (32-byte swizzle), the second group's
 // blocks in reverse order.
 __global__ void __launch_bounds__(kTriChunk * TNS) tri_coeff_kernel(TriArgs a, const int32_t* chunk_inst) {
@@ -897,7 +913,7 @@ __global__ void __launch_bounds__(kTriChunk * TNS) tri_coeff_kernel(TriArgs a, c
 #pragma unroll
   for (int i = 0; i < kTriChunk; ++i) mx = red[i][s] > mx ? red[i][s] : mx;
   const int ec = scale_exponent(mx);
-  if (kc == 0 && q == 0) d.cexp[g * TNS + s] = ec;
+  if (kc == 0 && q == 0) d.cexp[g * TNS + s] = ec + (src && ec != kNonFiniteRow ? d.cexp[g * TNS + s] : 0);
   const int64_t pos = kc * kTriChunk + q;
   double c = 0.0;
   if (s < d.S && ec != kNonFiniteRow) {
