@@ -316,6 +316,7 @@ __device__ __forceinline__ int scale_of(double most) {
 }
 // n_max <= 3 (tiles of one chunk): the polynomials themselves, for the digit warps too.
 __device__ __forceinline__ int row_scale_low(double rho, int n_max) {
+  if (!isfinite(rho)) return kNonFiniteRow;  // also of n_max = 0, which has no polynomial of rho below
   double most = 1.0;
   const double u = rho * rho, R[5] = {rho, fma(2.0, u, -1.0), u, rho * fma(3.0, u, -2.0), rho * u};
   const int n_of[5] = {1, 2, 2, 3, 3};
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
     const int64_t p = p0 + row;
     const bool valid = p < d.P;
     rho = valid ? d.r[p] : 0.0;
-    th = valid ? d.theta[p] : 0.0;
+    th = valid && d.n_max > 0 ? d.theta[p] : 0.0;  // a constant has no angle, also none that is not finite
     const uint32_t e = ((uint32_t)__double2hiint(th) >> 20) & 0x7ffu;
     return __any_sync(0xffffffffu, !(rho >= 0.0 && rho <= 1.0 && e < (uint32_t)kTriAngleExponent));
   };
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
       bool zero_row = false;  // float64 walk: a non-finite row, and the row's scale
       int shift = 0;
       auto set_scale = [&](int E) {
-        zero_row = E == kNonFiniteRow || (n_max > 0 && !isfinite(th));
+        zero_row = E == kNonFiniteRow || !isfinite(th);
         cur.ep = zero_row ? kNonFiniteRow : E;
         shift = kRowScale - (zero_row ? 0 : E);
       };

@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(WIDE ? kWideWarps * W : W) tri_walk_kernel(Tri
         }
       };
       element(e00, u0, l0, dg, nd0);
+      if (A == 0) e00[0] = 1.0;  // R_0^0, also of a radius that is not finite (0 rho would not be)
       element(e01, u1, e00, u0, nd1);
       element(e10, e00, l1, l0, nd1);
       element(e11, e01, e10, e00, nd2);
