@@ -24,8 +24,10 @@ from . import _lib
 PREC = {"fp64": 0, "bf16x3": 1, "tf32": 2, "fp64emu": 4}
 
 
-# The stream pointer without building a torch.cuda.Stream (2 us of a small call's 16 us of host time).
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# The stream pointer without building a torch.cuda.Stream (2 us of a small call's 16 us of host time),
+# where torch has that function (a build without CUDA does not).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
 
 
 def _stream(device: torch.device) -> int:
