@@ -19,20 +19,30 @@ __device__ __forceinline__ double from_fixed62(int64_t v) {
 // The same as a float32 (24 bits of the larger part).
 __device__ __forceinline__ float from_split62(const TriTrig& t) { return fmaf((float)t.lo, 0x1p-62f, (float)t.hi * 0x1p-31f); }
 
-// Calls f(m, cos m theta, sin m theta) for m = 0 .. m_max, in T.  In fixed point (absolute errors below 2^-57;
-// a float64 product m theta alone rounds by up to 2^-53 m theta) unless the angle is so small that
-// sin(m theta) needs relative accuracy, or out of range: then by angle addition in float64, restarted
-// from sincos at every 16th m.  (For float32 results fixed point serves as long as neither cos theta
-// nor sin theta is below 2^-36: 26 bits of either are left.)
+// cos and sin of m theta: of the rounded product, turned by what its rounding leaves out (a part of 2^-53 m theta,
+// which next to an axis would be all that is left).
+__device__ __forceinline__ void sincos_multiple(int m, double th, double* s, double* c) {
+  const double p = (double)m * th, e = fma((double)m, th, -p);
+  double s0, c0;
+  sincos(p, &s0, &c0);
+  *s = fma(e, c0, s0);
+  *c = fma(-e, s0, c0);
+}
+
+// Calls f(m, cos m theta, sin m theta) for m = 0 .. m_max, in T.  In fixed point, with absolute errors below
+// (m + 1) 2^-58 (2^-55 measured at m = 32, 2^-53 at 128; a float64 product m theta alone rounds by up to
+// 2^-53 m theta), unless the angle is out of range or so close to a multiple of a quarter turn that
+// cos or sin of its multiples need relative accuracy: then by angle addition in float64, restarted from
+// sincos at every 16th m.  The line: cos and sin both at least 2^-9 (53 bits in fixed point; a quarter of
+// a percent of all angles are closer), for float32 results 2^-36 (26 bits).
 template <typename T = double, typename F>
 __device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
   constexpr bool kFloat = sizeof(T) == sizeof(float);
-  const double mag = fabs(th);
   int64_t ci = 0, si = 0;
-  bool fixed = mag < 2048.0 && (kFloat || mag >= 1.0 / 128);
+  bool fixed = fabs(th) < 2048.0;
   if (fixed) {
     tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
-    if constexpr (kFloat) fixed = min(llabs(ci), llabs(si)) >= 1ll << 26;
+    fixed = tri_off_axes(ci, si, kFloat ? 26 : 53);
   }
   if (fixed) {
     const TriTrig c1 = tri_split(ci), s1 = tri_split(si);
@@ -52,7 +62,7 @@ __device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
     sincos(th, &s1, &c1);
     for (int m = 0; m <= m_max; ++m) {
       if (m % 16 == 0) {
-        if (m > 0) sincos((double)m * th, &s, &c);
+        if (m > 0) sincos_multiple(m, th, &s, &c);
       } else {
         const double cn = fma(c, c1, -s * s1);
         s = fma(s, c1, c * s1);

@@ -153,10 +153,10 @@ __global__ void __launch_bounds__(TPB) walk_kernel(WalkArgs a) {
         }
       }
     } else if (m != 0) {
-      sincos((double)m * a.theta[p0], &sn[0], &cs[0]);
+      sincos_multiple(m, a.theta[p0], &sn[0], &cs[0]);
       if constexpr (PPT == 2) {
         const double th1 = two ? a.theta[p0 + 1] : 0.0;
-        sincos((double)m * th1, &sn[PPT - 1], &cs[PPT - 1]);
+        sincos_multiple(m, th1, &sn[PPT - 1], &cs[PPT - 1]);
       }
     }
   }
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(TPB) walk_unweighted_kernel(WalkArgs a) {
       c = a.cs[(int64_t)m * a.P + p];
       s = a.sn[(int64_t)m * a.P + p];
     } else if (m != 0) {
-      sincos((double)m * a.theta[p], &s, &c);
+      sincos_multiple(m, a.theta[p], &s, &c);
     }
     if (a.pw != nullptr) {
       pm = a.pw[(int64_t)m * a.P + p];
