@@ -39,7 +39,7 @@ template <typename T = double, typename F>
 __device__ __forceinline__ void for_each_angle(double th, int m_max, F&& f) {
   constexpr bool kFloat = sizeof(T) == sizeof(float);
   int64_t ci = 0, si = 0;
-  bool fixed = fabs(th) < 2048.0;
+  bool fixed = fabs(th) < 0x1p52;
   if (fixed) {
     tri_cos_sin(tri_turn((uint64_t)__double_as_longlong(th)), ci, si);
     fixed = tri_off_axes(ci, si, kFloat ? 26 : 53);

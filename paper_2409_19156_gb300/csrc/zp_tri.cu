@@ -31,7 +31,7 @@
 //  - warps 0-7 drain finished accumulators.  One group: two accumulators, the previous segment
 //    drained after the next is produced.  Two groups (gradients): both accumulators hold one
 //    tile, drained before the next tile's first chunk.
-// Points off the unit disc (or at angles beyond 2^11) make their quadrant take the same walk in
+// Points off the unit disc (or at angles of 2^52 and more) make their quadrant take the same walk in
 // float64, with a row scale of its own per point.
 //
 // Bound: the integer instructions of the digit warps and their latencies (issue slots 55 %, ALU pipe

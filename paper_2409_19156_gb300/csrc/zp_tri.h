@@ -193,9 +193,9 @@ __host__ __device__ __forceinline__ int64_t tri_mul(const TriTrig& a, const TriT
   return (int64_t)a.hi * b.hi + (mid >> 31);
 }
 
-// A float64 angle, |theta| < 2^11, as a fraction of a turn at scale 2^64 (whole turns dropped):
-// theta times 126 bits of 1 / (2 pi).  Multiples of the angle are multiples of the word.
-constexpr int kTriAngleExponent = 1023 + 11;  // biased exponents below it
+// A float64 angle, |theta| < 2^52, as a fraction of a turn at scale 2^64 (whole turns dropped):
+// theta times 128 bits of 1 / (2 pi), within 1.5 units.  Multiples of the angle are multiples of the word.
+constexpr int kTriAngleExponent = 1023 + 52;  // biased exponents below it
 __host__ __device__ __forceinline__ uint64_t tri_turn(uint64_t theta_bits) {
   const int e = (int)((theta_bits >> 52) & 0x7ffu);
   const uint64_t mant = e ? (theta_bits & 0xfffffffffffffull) | (1ull << 52) : 0ull;
@@ -203,7 +203,7 @@ __host__ __device__ __forceinline__ uint64_t tri_turn(uint64_t theta_bits) {
   constexpr uint64_t kI1 = 0x28be60db9391054aull, kI0 = 0x7f09d5f47d4d3770ull;
   const uint64_t p0 = mant * kI1, q0 = tri_umul_hi(mant, kI0);
   const uint64_t ql = p0 + q0, qh = tri_umul_hi(mant, kI1) + (ql < p0 ? 1u : 0u);
-  const int sh = 1075 - e;  // turn = (qh 2^64 + ql) 2^-sh mod 2^64; sh >= 42
+  const int sh = 1075 - e;  // turn = (qh 2^64 + ql) 2^-sh mod 2^64; sh >= 1
   const uint64_t turn = sh < 64 ? (qh << (64 - sh)) | (ql >> sh) : (sh < 128 ? qh >> (sh - 64) : 0ull);
   return theta_bits >> 63 ? 0 - turn : turn;
 }
@@ -252,8 +252,8 @@ __host__ __device__ __forceinline__ bool tri_off_axes(int64_t c, int64_t s, int 
   return ((ac < as ? ac : as) >> bits) != 0;
 }
 
-// The next angle of a table: (c, s) turned by (c1, s1).  The m-th is within (m + 1) 10 2^-62: of that 1.6 per m
-// from the word of the turn, 4 of the first angle's own, and two truncated products.
+// The next angle of a table: (c, s) turned by (c1, s1).  The m-th is within (m + 1) 10 2^-62: of that up to 2.4
+// per m from the word of the turn, 4 of the first angle's own, and two truncated products.
 __host__ __device__ __forceinline__ void tri_rotate(TriTrig& c, TriTrig& s, const TriTrig& c1, const TriTrig& s1) {
   const int64_t cn = tri_mul(c, c1) - tri_mul(s, s1);
   const int64_t sn = tri_mul(s, c1) + tri_mul(c, s1) + 1;

@@ -23,6 +23,7 @@ def test_table_against_oracle(tmp_path):
                    check=True, capture_output=True)
     axes = [q * np.pi / 2 + d for q in (-1, 0, 1, 2, 3, 4, 100) for d in (0.0, 1e-9, -1e-4, 1.9e-3)]
     off = list(np.random.default_rng(0).uniform(-2000.0, 2000.0, 12)) + [q * np.pi / 2 + 2.1e-3 for q in (0, 1, 2, 3)]
+    off += [2047.5, 2100.0, -5000.0, 1e6, 1e9, -3.0e12, 2.0 ** 51 + 0.5, 2.0 ** 52 - 0.5]  # large angles too
     text = "".join(f"{float(t).hex()}\n" for t in axes + off)
     lines = [[int(x) for x in line.split()] for line in subprocess.run(
         [exe, str(m_max)], input=text, capture_output=True, text=True, check=True).stdout.splitlines()]
@@ -51,3 +52,27 @@ def test_functions_next_to_the_axes():
             # m theta is next to an axis too: cos and sin are near +-1 or near m times the distance, with one
             # sign in every sum.  Angle addition rounds each factor twice per step, R twice per value.
             assert (np.abs(got[j] - want) <= 8 * (abs(m) + 1) * 2.0 ** -53 * np.abs(want)).all(), (k, m)
+
+
+@pytest.mark.gpu
+def test_series_at_large_angles():
+    """Angles up to 2^52 against the oracle: the fused series, its gradients and the split basis."""
+    torch = pytest.importorskip("torch")
+    import paper_2409_19156_gb300 as zp
+    from oracle import basis as obasis
+
+    ns, ms = inputs.full_zernike_modes(20)
+    th = np.array([2047.0, 2048.0, -2049.0, 5000.25, 1e6, -1e9, 3.0e12, 2.0 ** 51 + 0.5, 2.0 ** 52 - 0.5, 2.0 ** 52, 1e17])
+    r = np.linspace(0.1, 1.0, len(th))
+    C = inputs.scaled_normal_coeffs(ns, 3, 5)
+    z, zt = (np.array(x) for x in obasis.basis_table(ns, ms, r, th, 1, with_dtheta=True))
+    plan, G = zp.Plan(ns, ms), np.ones((len(th), 3))
+    rt, tt, Ct, Gt = (torch.as_tensor(x, device="cuda") for x in (r, th, C, G))
+    F = zp.series_eval(None, None, rt, tt, Ct, plan=plan).cpu().numpy()
+    size = np.abs(C).sum(0)
+    assert (np.abs(F - z[0].T @ C) <= 1e-13 * (1.0 + size)).all()
+    gr, gt = (x.cpu().numpy() for x in zp.series_adjoint(None, None, rt, tt, Ct, Gt, need=(False, True, True), plan=plan)[1:])
+    for got, d in ((gr, z[1]), (gt, zt)):  # derivatives of up to n^2 <= 400 per mode
+        assert (np.abs(got - (d.T @ C).sum(1)) <= 1e-13 * (1.0 + 400.0 * size.sum())).all()
+    got = zp.series_eval(None, None, rt, tt, Ct, prec="bf16x3", plan=plan).double().cpu().numpy()
+    assert (np.abs(got - z[0].T @ C) <= 1e-4 * (np.abs(z[0]).T @ np.abs(C))).all()
