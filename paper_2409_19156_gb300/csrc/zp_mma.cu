@@ -374,7 +374,7 @@ struct TriBasisArgs {
 };
 
 __host__ __device__ constexpr uint32_t tri_basis_smem(int n_max) {
-  return (uint32_t)((2 * (n_max / 4) + 2) * BM * 8 + (n_max + 1) * BM * 8 + (tri_blocks(n_max) + 15) / 16 * 16);
+  return (uint32_t)(tri_state_rows(n_max) * BM * 8 + (n_max + 1) * BM * 8 + (tri_blocks(n_max) + 15) / 16 * 16);
 }
 // Two blocks or more per SM.
 constexpr uint32_t kTriBasisSmem = 110 * 1024;
@@ -447,8 +447,8 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
       l0 = e01;
       l1 = e11;
       const float f[4] = {e00.x + e00.y, e01.x + e01.y, e10.x + e10.y, e11.x + e11.y};
-      const int m0 = 2 * (A - B);
-      const float2 mid = an[(size_t)m0 * BM], low = an[(size_t)max(m0 - 1, 0) * BM], top = an[(size_t)min(m0 + 1, n_max) * BM];
+      const TriAngleRows am = tri_angle_rows(2 * (A - B), n_max);
+      const float2 mid = an[(size_t)am.mid * BM], low = an[(size_t)am.low * BM], top = an[(size_t)am.top * BM];
       const float z[8] = {f[0] * mid.x, f[1] * low.x, f[2] * top.x, f[3] * mid.x,
                           f[0] * mid.y, f[1] * low.y, f[2] * top.y, f[3] * mid.y};
       if (whole[block]) {
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(BM) tri_basis_kernel(TriBasisArgs a) {
   using C = Cfg<TF32 ? KIND_TF32 : KIND_BF16X3>;
   extern __shared__ float2 tri_basis_mem[];
   float2* st = tri_basis_mem + threadIdx.x;
-  float2* angles = tri_basis_mem + (size_t)(2 * (a.n_max / 4) + 2) * BM;
+  float2* angles = tri_basis_mem + (size_t)tri_state_rows(a.n_max) * BM;
   float2* an = angles + threadIdx.x;
   // Which blocks have all their modes (a load per block would stall on its latency).
   uint8_t* whole = reinterpret_cast<uint8_t*>(angles + (size_t)(a.n_max + 1) * BM);

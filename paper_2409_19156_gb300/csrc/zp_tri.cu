@@ -88,8 +88,7 @@ constexpr int kRowScale = 62;                // a value of row scale E is digiti
 // second group's digits in reverse order, 8 zero blocks, the first group's digits, so that both
 // share the zero blocks (the second group's accumulator then holds its diagonals in reverse).
 __host__ __device__ constexpr uint32_t stage_bytes(int groups) { return kZeroB + (uint32_t)groups * kTriGroupBytes; }
-__host__ __device__ constexpr int state_rows(int n_max) { return 2 * (n_max / 4) + 2; }
-__host__ __device__ constexpr uint32_t state_bytes(int n_max) { return (uint32_t)state_rows(n_max) * TM * 8u; }
+__host__ __device__ constexpr uint32_t state_bytes(int n_max) { return (uint32_t)tri_state_rows(n_max) * TM * 8u; }
 __host__ __device__ constexpr uint32_t angle_bytes(int n_max) { return (uint32_t)(n_max + 1) * TM * 16u; }
 __host__ __device__ constexpr uint32_t smem_bytes(int n_max, int groups, int stages) {
   return 256u + kAux + (groups == 2 ? kSwapB : 0u) + kRingB + state_bytes(n_max) + angle_bytes(n_max) +
@@ -294,17 +293,6 @@ __device__ __forceinline__ bool drain_segment(const TriArgs& a, const Pending& p
   }
   return true;
 }
-
-// The order of a tile's blocks: row A, block B of 0 .. nb.
-struct BlockIndex {
-  int A = 0, B = 0, nb = 0;
-  __device__ __forceinline__ void advance(int H) {
-    const bool end = B == nb;
-    A += end;
-    B = end ? 0 : B + 1;
-    nb = min(A, H - A);
-  }
-};
 
 // Row scale exponent of a point walked in float64: 2^E above 1.02 times the largest |R| of its
 // triangle (the margin keeps the leading digit's field within seven bits); kNonFiniteRow when a
@@ -528,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
       }
 
       const uint32_t lane_base = tmem_base + ((quad * 32u) << 16) + kABase;
-      BlockIndex bi;
+      TriBlock bi;
       int seg_left = seg_chunks;
       for (int kc = 0; kc < KC; ++kc) {
         if (turn_of == group) {
@@ -546,10 +534,8 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
             ptx::tc_fence_after();
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-              const int m0 = 2 * (bi.A - bi.B);
-              const ulonglong2 mid = an[(size_t)min(m0, n_max) * TM];
-              const ulonglong2 low = an[(size_t)min(max(m0 - 1, 0), n_max) * TM];
-              const ulonglong2 top = an[(size_t)min(m0 + 1, n_max) * TM];
+              const TriAngleRows am = tri_angle_rows(2 * (bi.A - bi.B), n_max);
+              const ulonglong2 mid = an[(size_t)am.mid * TM], low = an[(size_t)am.low * TM], top = an[(size_t)am.top * TM];
               uint32_t wc0[TND], wc1[TND], ws0[TND], ws1[TND];
               const uint64_t mc = tri_offset(mid.x), ms = tri_offset(mid.y);
               digits_of(tri_word(v[4 * k], mid.x, mc), tri_word(v[4 * k + 1], low.x, tri_offset(low.x)), wc0, dc);
@@ -568,15 +554,16 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
             ptx::tc_fence_after();
 #pragma unroll 1
             for (int k = 0; k < 2; ++k) {
-              const int m0 = 2 * (bi.A - bi.B), n0 = 2 * (bi.A + bi.B);
+              const TriAngleRows am = tri_angle_rows(2 * (bi.A - bi.B), n_max);
+              const int n0 = 2 * (bi.A + bi.B);
               uint32_t w[4][TND];
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 uint64_t y[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                  const int m = m0 + (e == 1 ? -1 : e == 2 ? 1 : 0), n = n0 + (e == 0 ? 0 : e == 3 ? 2 : 1);
-                  const ulonglong2 g = an[(size_t)min(max(m, 0), n_max) * TM];
+                  const int n = n0 + (e == 0 ? 0 : e == 3 ? 2 : 1);
+                  const ulonglong2 g = an[(size_t)(e == 1 ? am.low : e == 2 ? am.top : am.mid) * TM];
                   const double z = __longlong_as_double((long long)f[(size_t)(4 * k + e) * TM]) *
                                    __longlong_as_double((long long)(h ? g.y : g.x));
                   // Elements above n_max (and all of a non-finite row) have no coefficients: zero.
@@ -644,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
       const bool slow = point_of(d, p0, rho, th);
       const TriPoint tp = tri_point((uint64_t)__double_as_longlong(rho));
       const int scale = slow && KC > 1 ? row_scale(rho, n_max, st) : 0;
-      BlockIndex bi;
+      TriBlock bi;
       uint64_t l0 = 0, l1 = 0, dg = 0;  // f(2A, 2B-1), f(2A+1, 2B-1), f(2A-1, 2B-1): biased words or float64 bits
       for (int kc = 0; kc < KC; ++kc) {
         ok = warp_wait(&bar->rempty[slot][quad], rphase ^ 1u, abort_flag, lane);

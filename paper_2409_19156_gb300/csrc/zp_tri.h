@@ -78,6 +78,29 @@ __host__ __device__ constexpr void tri_mode(int p, int n_max, int& n, int& m, in
   sine = (p >> 2) & 1;
 }
 
+// The order of a point's blocks: row A, block B of 0 .. nb.  An odd number of blocks leaves the last chunk
+// one more, past the last row (B = 0): its values have no modes.
+struct TriBlock {
+  int A = 0, B = 0, nb = 0;
+  __host__ __device__ __forceinline__ void advance(int H) {
+    const bool end = B == nb;
+    A += end;
+    B = end ? 0 : B + 1;
+    nb = A < H - A ? A : H - A;
+  }
+};
+// Rows of the stored row above (two per block).
+__host__ __device__ constexpr int tri_state_rows(int n_max) { return 2 * (n_max / 4) + 2; }
+// Rows of an angle table [0, n_max] for a block of |m| = m0 - 1 (e01), m0 (e00, e11) and m0 + 1 (e10), m0 >= 0;
+// elements without a mode take a row that exists.
+struct TriAngleRows {
+  int low, mid, top;
+};
+__host__ __device__ __forceinline__ TriAngleRows tri_angle_rows(int m0, int n_max) {
+  const int low = m0 > 0 ? m0 - 1 : 0;
+  return {low < n_max ? low : n_max, m0 < n_max ? m0 : n_max, m0 + 1 < n_max ? m0 + 1 : n_max};
+}
+
 // ------------------------------------------------------------------ arithmetic (host and device)
 
 __host__ __device__ __forceinline__ uint64_t tri_umul_hi(uint64_t a, uint64_t b) {

@@ -55,20 +55,19 @@ struct TriWalkArgs {
   int n_max;
 };
 
-__host__ __device__ constexpr int rows_of(int n_max) { return 2 * (n_max / 4) + 2; }
 __host__ __device__ constexpr uint32_t walk_smem(int n_max, int kmax, bool ang) {
-  return (uint32_t)(rows_of(n_max) * (kmax + 1) * W * 8 + (n_max + 3) * 8 + (ang ? (n_max + 1) * W * 16 : 0));
+  return (uint32_t)(tri_state_rows(n_max) * (kmax + 1) * W * 8 + (n_max + 3) * 8 + (ang ? (n_max + 1) * W * 16 : 0));
 }
 
 constexpr uint32_t wide_smem(int n_max, int kmax) {
-  return (uint32_t)(rows_of(n_max) * (kmax + 1 - kWideLanes) * kWideWarps * W * 8 + (n_max + 3) * 8);
+  return (uint32_t)(tri_state_rows(n_max) * (kmax + 1 - kWideLanes) * kWideWarps * W * 8 + (n_max + 3) * 8);
 }
 // Whether the wide form fits (tensor memory columns and shared memory of one block per SM) and the
 // one-warp form leaves fewer than six warps per SM (1e5 points, wide against one-warp form: k <= 3, four
 // per SM, n <= 100: 3.71 against 4.62 ms; five per SM, n <= 72, k <= 3: 2.02 against 2.14 ms, and n <= 100,
 // k <= 2: 2.80 against 2.91 ms).
 constexpr bool wide_fits(int n_max, int kmax, bool ang) {
-  return !ang && kmax >= 2 && rows_of(n_max) * kWideLanes * 2 <= kWideCols && wide_smem(n_max, kmax) <= kMaxBlockSmem &&
+  return !ang && kmax >= 2 && tri_state_rows(n_max) * kWideLanes * 2 <= kWideCols && wide_smem(n_max, kmax) <= kMaxBlockSmem &&
          walk_smem(n_max, kmax, false) + kSmemPerBlock > kSmemPerSm / 6;
 }
 
@@ -86,8 +85,8 @@ __global__ void __launch_bounds__(WIDE ? kWideWarps * W : W) tri_walk_kernel(Tri
   constexpr int kUnroll = ANG ? 1 : 4;
   const int lane = threadIdx.x % W, warp = threadIdx.x / W, n_max = a.n_max, H = n_max / 2;
   double2* an = reinterpret_cast<double2*>(tri_smem) + lane;  // [m][lane]
-  double* st = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)warp * rows_of(n_max) * LS * W + lane;  // [b][k][lane]
-  double* num = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)kWarps * rows_of(n_max) * LS * W;  // 0, 1, 2, ..
+  double* st = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)warp * tri_state_rows(n_max) * LS * W + lane;  // [b][k][lane]
+  double* num = tri_smem + (ANG ? (size_t)(n_max + 1) * W * 2 : 0) + (size_t)kWarps * tri_state_rows(n_max) * LS * W;  // 0, 1, 2, ..
   for (int i = threadIdx.x; i < n_max + 3; i += kWarps * W) num[i] = (double)i;
   uint32_t tm = 0;  // [b / 2][row of two][k][low, high word] of this thread's lane
   if constexpr (WIDE) {
@@ -224,10 +223,11 @@ __global__ void __launch_bounds__(WIDE ? kWideWarps * W : W) tri_walk_kernel(Tri
         ptx::tmem_st_32x32b_x4<0>(tm + 8 * B, lo(e10[LS]), hi(e10[LS]), lo(e10[LS + 1]), hi(e10[LS + 1]));
         ptx::tmem_st_32x32b_x4<4>(tm + 8 * B, lo(e11[LS]), hi(e11[LS]), lo(e11[LS + 1]), hi(e11[LS + 1]));
       }
-      emit(e00, jc.x, js.x, m0);
-      emit(e01, jc.y, js.y, max(m0 - 1, 0));
-      emit(e10, jc.z, js.z, min(m0 + 1, n_max));
-      emit(e11, jc.w, js.w, m0);
+      const TriAngleRows am = tri_angle_rows(m0, n_max);
+      emit(e00, jc.x, js.x, am.mid);
+      emit(e01, jc.y, js.y, am.low);
+      emit(e10, jc.z, js.z, am.top);
+      emit(e11, jc.w, js.w, am.mid);
     }
     if constexpr (WIDE) {  // before the next row's reads
       __syncwarp();
