@@ -294,6 +294,38 @@ __device__ __forceinline__ bool drain_segment(const TriArgs& a, const Pending& p
   return true;
 }
 
+// A chunk's digits from values walked in float64, digitised at the row's scale.  Out of line, so that the
+// fixed-point digits' registers and code are not laid out around it: 1e6 points on the disc, n <= 32, 16 sets
+// 2.41 -> 2.32 ms; a 1000 x 1000 pixel grid with a fifth of its points off the disc 4.29 -> 4.46 ms.
+__device__ __noinline__ void digits_of_float64(const uint64_t* f, const ulonglong2* an, TriBlock bi, int n_max, bool zero_row,
+                                               int shift, uint32_t at, DigitConst dc) {
+  const int H = n_max / 2;
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const TriAngleRows am = tri_angle_rows(2 * (bi.A - bi.B), n_max);
+    const int n0 = 2 * (bi.A + bi.B);
+    uint32_t w[4][TND];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint64_t y[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int n = n0 + (e == 0 ? 0 : e == 3 ? 2 : 1);
+        const ulonglong2 g = an[(size_t)(e == 1 ? am.low : e == 2 ? am.top : am.mid) * TM];
+        const double z = __longlong_as_double((long long)f[(size_t)(4 * k + e) * TM]) *
+                         __longlong_as_double((long long)(h ? g.y : g.x));
+        // Elements above n_max (and all of a non-finite row) have no coefficients: zero.
+        y[e] = (uint64_t)(zero_row || n > n_max ? 0 : to_fixed(z, shift)) + kTriWordBias;
+      }
+      digits_of(y[0], y[1], w[2 * h], dc);
+      digits_of(y[2], y[3], w[2 * h + 1], dc);
+    }
+    __syncwarp();  // to_fixed parts the lanes; a tensor-memory store is the whole warp's
+    store_digits(at + 4u * k, w[0], w[1], w[2], w[3]);
+    bi.advance(H);
+  }
+}
+
 // Row scale exponent of a point walked in float64: 2^E above 1.02 times the largest |R| of its
 // triangle (the margin keeps the leading digit's field within seven bits); kNonFiniteRow when a
 // value is not finite.
@@ -552,30 +584,9 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
             ok = warp_wait(&bar->empty[stage], sphase ^ 1u, abort_flag, lane);
             if (!ok) break;
             ptx::tc_fence_after();
-#pragma unroll 1
-            for (int k = 0; k < 2; ++k) {
-              const TriAngleRows am = tri_angle_rows(2 * (bi.A - bi.B), n_max);
-              const int n0 = 2 * (bi.A + bi.B);
-              uint32_t w[4][TND];
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                uint64_t y[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const int n = n0 + (e == 0 ? 0 : e == 3 ? 2 : 1);
-                  const ulonglong2 g = an[(size_t)(e == 1 ? am.low : e == 2 ? am.top : am.mid) * TM];
-                  const double z = __longlong_as_double((long long)f[(size_t)(4 * k + e) * TM]) *
-                                   __longlong_as_double((long long)(h ? g.y : g.x));
-                  // Elements above n_max (and all of a non-finite row) have no coefficients: zero.
-                  y[e] = (uint64_t)(zero_row || n > n_max ? 0 : to_fixed(z, shift)) + kTriWordBias;
-                }
-                digits_of(y[0], y[1], w[2 * h], dc);
-                digits_of(y[2], y[3], w[2 * h + 1], dc);
-              }
-              __syncwarp();  // to_fixed parts the lanes; a tensor-memory store is the whole warp's
-              store_digits(lane_base + (uint32_t)stage * kAStage + 4u * k, w[0], w[1], w[2], w[3]);
-              bi.advance(H);
-            }
+            digits_of_float64(f, an, bi, n_max, zero_row, shift, lane_base + (uint32_t)stage * kAStage, dc);
+            bi.advance(H);
+            bi.advance(H);
           }
           ptx::tmem_st_wait();
           ptx::tc_fence_before();
