@@ -16,6 +16,10 @@
  *    Output columns follow the caller's mode order.  Radial entry points use |m|.
  *  - Point arrays r[] (and theta[]) are DEVICE float64 arrays of length n_points.  r is
  *    evaluated as the polynomial it is: values outside [0, 1] are not clamped.
+ *    A point's results may differ in their last bits with its place in the arrays and with
+ *    n_points: large calls split the points between kernels that round differently.  A point
+ *    that is not finite, or whose values overflow, gives outputs that are not finite (of the
+ *    constant mode too in a fused series) and leaves other points alone.
  *  - Outputs are DEVICE arrays owned and allocated by the caller; the library never keeps a
  *    pointer to them after the call returns.
  *  - DEVICE means reachable by the current device at that address: its own memory, managed
@@ -229,6 +233,10 @@ ZP_API zp_status zp_series_adjoint_plan(const zp_plan* plan, const double* r, co
  * reduced in float64 as for ZP_PREC_FP64 -- except for n_sets <= 16 (and at most 5041 padded
  * modes), where they are the row sums grad_out[p] . (dZ/dtheta C)[p] and grad_out[p] . (dZ/drho
  * C)[p] of the fused kernel's derivative series (no modes x points matrix H; deterministic).
+ * Mode lists that fill their triangle up to n = 64 take dF/dx and dF/dy as two series, then
+ * dF/dr = cos F_x + sin F_y and dF/dtheta = r (cos F_y - sin F_x): the error of either is measured
+ * by the whole gradient, so that the grad_theta of a rotationally symmetric surface is rounding
+ * noise of r dF/dr and not exactly 0.
  * Other precisions: ZP_ERR_INVALID_ARG.
  */
 ZP_API zp_status zp_series_adjoint_plan_prec(const zp_plan* plan, const double* r, const double* theta,
