@@ -389,8 +389,7 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
   rho = n_max > 0 ? rho : 0.0;
   for_each_angle<float>(th, n_max, [&](int m, float c, float s) { an[(size_t)m * BM] = make_float2(c, s); });
   const float rh = (float)rho, rl = isfinite(rh) ? (float)(rho - (double)rh) : 0.0f;
-  const PairFactor<float> r1{rh, -rh, -rl};
-  const PairFactor<f32x2> r2{f32x2::of(rh, rh), f32x2::of(-rh, -rh), f32x2::of(-rl, -rl)};
+  const float2 pair_rho = make_float2(rh, rl);
   int k_full = 0, k_tail = 8 * a.full;
   Pack16 hi, lo;
   auto at = [&](int k, uint32_t r) {  // a unit's place in row r
@@ -437,10 +436,9 @@ __device__ __forceinline__ void tri_basis_row(const TriBasisArgs& a, uint8_t* gA
     for (int B = 0; B <= nb; ++B, ++block) {
       float2* sr = st + (size_t)(2 * B) * BM;
       const float2 u0 = B < A ? sr[0] : l0, u1 = B < A ? sr[BM] : l1;
-      const float2 e00 = pair_step(r1, u0, l0, dg);
-      float2 e01, e10;  // independent of each other: one instruction for both
-      pair_step2(r2, u1, e00, u0, e00, l1, l0, e01, e10);
-      const float2 e11 = pair_step(r1, e01, e10, e00);
+      const float2 e00 = pair_step(pair_rho, u0, l0, dg);
+      const float2 e01 = pair_step(pair_rho, u1, e00, u0), e10 = pair_step(pair_rho, e00, l1, l0);
+      const float2 e11 = pair_step(pair_rho, e01, e10, e00);
       sr[0] = e10;
       sr[BM] = e11;
       dg = u1;

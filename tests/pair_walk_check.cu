@@ -16,7 +16,7 @@ int main(int, char** argv) {
   while (std::scanf("%63s", text) == 1) {
     const double rho = std::strtod(text, nullptr);
     const float rh = (float)rho, rl = (float)(rho - (double)rh);
-    const PairFactor<float> r{rh, -rh, -rl};
+    const float2 r = make_float2(rh, rl);
     std::vector<float2> st(2 * (n_max / 4) + 2);
     for (int A = 0; A <= H; ++A) {
       float2 l0 = make_float2(0.0f, 0.0f), l1 = l0, dg = make_float2(A == 0 ? -1.0f : 0.0f, 0.0f);
