@@ -42,9 +42,9 @@ DP_OPS_PEAK_NOMINAL = SMS * DP_LANES_PER_SM * SM_MAX_MHZ * 1e6
 # (4 FMA): 7 float64 operations, 11 flop.  (The column recursion it replaced takes 15, 28 flop.)
 FLOP_PER_VALUE_TUPLE = 11
 DP_OPS_PER_VALUE_TUPLE = 7
-# DRAM bytes (read + write) of one one-warp tri_walk_kernel<3,false,false,false> launch at 19456 points,
-# from one ncu capture (its output is 1.619 GB; the rest is in L2 at its end), scaled to 100000 points.
-WALK_TRAFFIC_POINTS, WALK_TRAFFIC = 19456, 1.557012224e9 + 0.217088e6
+# DRAM bytes (read + write) of one wide tri_walk_kernel<3,false,false,true> launch at 38912 points, from one
+# ncu capture (its output is 3.239 GB; the rest is in L2 at its end), scaled to 100000 points.
+WALK_TRAFFIC_POINTS, WALK_TRAFFIC = 38912, 3.176987904e9 + 0.432128e6
 
 
 def parse_args():
@@ -524,7 +524,7 @@ def run_ours(args) -> None:
             "roofline": {"bound": "alu", "achieved": achieved_flops / 1e12, "peak": peak_flops / 1e12,
                          "unit": "TFLOP/s", "frac": achieved_flops / peak_flops,
                          "traffic": WALK_TRAFFIC * P / WALK_TRAFFIC_POINTS if WALK_TRAFFIC else None,
-                         "traffic_note": "ncu dram__bytes_read+write of a 19456-point launch scaled by points",
+                         "traffic_note": "ncu dram__bytes_read+write of a 38912-point launch scaled by points",
                          "kernel": "tri_walk_kernel<3,false,false,true> (part waves: its one-warp form, walk_kernel)",
                          "flop_per_launch": flops,
                          "flop_per_unit": FLOP_PER_VALUE_TUPLE, "units_per_launch": P * J,

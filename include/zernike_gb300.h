@@ -138,7 +138,7 @@ ZP_API zp_status zp_radial_plan(const zp_plan* plan, const double* r, int64_t n_
 /*
  * zp_radial_plan with per-kernel timing: CUDA events are recorded on `stream` around each
  * launch and phase_ms[0] receives the device time of the point-preparation kernel (powers of
- * rho; 0 when the launch is too small to use it), phase_ms[1] that of the recursion walk.
+ * rho; 0 when the call does not use it: few points, or the walk over a filled triangle), phase_ms[1] that of the recursion walk.
  * Same outputs as zp_radial_plan.  The call synchronises `stream` before returning
  * (instrumentation; not for graph capture).
  */

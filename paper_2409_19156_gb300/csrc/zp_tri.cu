@@ -32,10 +32,13 @@
 //    drained after the next is produced.  Two groups (gradients): both accumulators hold one
 //    tile, drained before the next tile's first chunk.
 // Points off the unit disc (or at angles of 2^52 and more) make their quadrant take the same walk in
-// float64, with a row scale of its own per point.
+// float64, with a row scale of its own per point: a walk more, and three to four times the time.  A
+// 1000 x 1000 pixel grid over the square, n <= 32, 16 sets: 4.5 ms for values and 6.0 for gradients (the column
+// form 10.4 and 25.4); the same points in random order, where every quadrant has one off the disc, 8.1
+// and 8.3 (23.6 and 58.2).
 //
-// Bound: the integer instructions of the digit warps and their latencies (issue slots 55 %, ALU pipe
-// 52 %, tensor pipe 31 % busy).  1e6 points r = sqrt(U), 561 modes, 16 sets: 2.37 ms, against 3.91 ms
+// Bound: the integer instructions of the digit warps and their latencies (issue slots 56 %, ALU pipe
+// 55 %, tensor pipe 31 % busy).  1e6 points r = sqrt(U), 561 modes, 16 sets: 2.30 ms, against 3.91 ms
 // of the float64 column walk in zp_fused.cu, with a quarter of its error; both point gradients of
 // 300007 such points in one pass instead of two.  Measured on the way there: eight warps that each
 // walk and cut, one cos and one sin warp per quadrant 3.3 ms, with the multiplications in unsigned

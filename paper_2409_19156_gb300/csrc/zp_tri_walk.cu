@@ -17,8 +17,9 @@
 // With the whole row in shared memory, high degrees leave room for one warp per scheduler, which
 // keeps the pipe two thirds busy: the instructions between two float64 operations are not hidden.
 // The wide form (radial, k >= 2) holds the row's two highest derivative lanes in tensor memory (each
-// warp reads its own 32 lanes of it), so that two warps per scheduler fit: eight in a block, one
-// block per SM.
+// warp reads its own 32 lanes of it), so that two warps per scheduler fit: eight in a block that takes
+// all of tensor memory, so one block per SM works at a time (where shared memory admits another, it waits
+// for the first one's tensor memory).  Its float64 pipe is 90 % busy over whole waves.
 //
 // Measured against the column form: radial set n <= 100, k <= 3, 1e5 points 6.32 -> 3.66 ms (4.62
 // with one warp per scheduler); Z and dZ/drho with dZ/dtheta, n <= 32, 99991 points 836 -> 631 us.
