@@ -98,6 +98,7 @@ struct zp_plan {
   int32_t fused_units = 0;  // global 8-value units G of the layout (whole 4-unit stages); stream s owns (G - s + S - 1) / S
   int32_t fused_ep = 1;              // row scale exponent of the fused kernel on the unit disc
   bool tri = false;                  // the fused series takes the triangle layout (zp_tri.h)
+  bool tri_angles = false;           // some mode has m != 0
   std::vector<int32_t> tri_perm;     // the layout's positions' modes (empty without it)
   std::vector<int32_t> tri_order;    // modes in the split basis's K order: whole blocks, then the others
   int32_t tri_full = 0;              // whole blocks: all of their eight positions have modes

@@ -308,9 +308,8 @@ zp_status build_plan_host(const int32_t* n, const int32_t* m, int64_t n_modes, z
     // The fused series also wants enough of the positions taken.  A full list has about as many in
     // either layout, and there the triangle form takes 0.60 of the column form's time (n <= 32, 1e6
     // points, 16 sets: 2.37 against 3.91 ms), so up to half as many positions again still gain.
-    // (Lists of m = 0 alone keep the column form, whose outputs do not involve theta at all.)
-    const bool angles = n_max == 0 || std::any_of(m, m + n_modes, [](int32_t x) { return x != 0; });
-    p->tri = once && angles && n_max <= kTriMaxN && 2 * positions <= 3 * p->fused_kpad;
+    p->tri = once && n_max <= kTriMaxN && 2 * positions <= 3 * p->fused_kpad;
+    p->tri_angles = std::any_of(m, m + n_modes, [](int32_t x) { return x != 0; });
   }
   return ZP_OK;
 }

@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_kernel(TriArgs a, int n_max_l
     const int64_t p = p0 + row;
     const bool valid = p < d.P;
     rho = valid ? d.r[p] : 0.0;
-    th = valid && d.n_max > 0 ? d.theta[p] : 0.0;  // a constant has no angle, also none that is not finite
+    th = valid && d.theta ? d.theta[p] : 0.0;
     const uint32_t e = ((uint32_t)__double2hiint(th) >> 20) & 0x7ffu;
     return __any_sync(0xffffffffu, !(rho >= 0.0 && rho <= 1.0 && e < (uint32_t)kTriAngleExponent));
   };
@@ -983,7 +983,7 @@ TriInst tri_inst(const zp_plan* plan, const double* r, const double* theta, int6
   d.P = P;
   d.S = S;
   d.r = r;
-  d.theta = theta;
+  d.theta = plan->tri_angles ? theta : nullptr;  // outputs without angles take any theta
   d.coeffs = coeffs;
   d.perm = plan->dev.tri_perm;
   return d;

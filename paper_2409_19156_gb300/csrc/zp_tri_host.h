@@ -20,7 +20,7 @@ struct TriInst {
   int64_t kc_base = 0;     // first chunk in the launch's chunk numbering
   int64_t J = 0, P = 0, S = 0;
   const double* r = nullptr;
-  const double* theta = nullptr;
+  const double* theta = nullptr;    // NULL: no mode has an angle
   const double* coeffs = nullptr;   // [J][S]
   const int32_t* perm = nullptr;    // [KC * 16]: mode of every position, -1 for none
   uint8_t* bdig = nullptr;          // [KC][groups] digits (written per call)

@@ -58,3 +58,22 @@ def test_lists_without_angles_take_any_theta():
     assert torch.allclose(out, 3.0 - 2.0 * r * r, rtol=0.0, atol=2.0 ** -50)
     _, gr, gt = zp.series_adjoint([0, 2], [0, 0], r, th, C, torch.ones((70, 1), dtype=torch.float64, device="cuda"))
     assert torch.allclose(gr, -4.0 * r, rtol=0.0, atol=2.0 ** -49) and bool((gt == 0.0).all())
+
+
+def test_batch_with_a_list_without_angles():
+    """Beside full sets, with any theta: the same bits as alone."""
+    recs = []
+    for ns, ms, P in (([0, 2], [0, 0], 150), (*inputs.full_zernike_modes(11), 300), ([0], [0], 40)):
+        r, th = (torch.as_tensor(x, device="cuda") for x in inputs.uniform_points(P, P))
+        if max(np.abs(ms)) == 0:
+            th[::3] = float("nan")
+        C = torch.as_tensor(np.random.default_rng(P).standard_normal((len(ns), 2)), device="cuda")
+        recs.append({"n": ns, "m": ms, "r": r, "theta": th, "coeffs": C, "grad_out": torch.ones((P, 2), dtype=torch.float64, device="cuda")})
+    batch = zp.Batch(recs, 2)
+    batch.forward()
+    batch.adjoint()
+    for d, b in zip(recs, batch.instances):
+        args = (d["n"], d["m"], d["r"], d["theta"], d["coeffs"])
+        assert torch.equal(b["out"], zp.series_eval(*args)) and bool(torch.isfinite(b["out"]).all())
+        for got, want in zip((b["grad_r"], b["grad_theta"]), zp.series_adjoint(*args, d["grad_out"], need=(False, True, True))[1:]):
+            assert torch.equal(got, want) and bool(torch.isfinite(got).all())
